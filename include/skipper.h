@@ -77,9 +77,9 @@ typedef struct mm_options {
                                 32: one word per vertex that is also the mate
                                 entry (ACC = MM_UNMATCHED, RSVD = 0xFFFFFFFE,
                                 matched = partner id).  0 = 8. */
-    uint32_t serial;         /* 1: one GPU thread walks rows in ascending order and
+    uint32_t serial;         /* 1: one warp walks rows in ascending order and
                                 neighbours in stored order (per graph in batched
-                                mode); the result equals sequential greedy MM. */
+                                mode; an edge list: one thread); the result equals sequential greedy MM. */
     uint32_t grain;          /* merge-path items (rows + entries; edges for an edge
                                 list) per work unit.  Must be a multiple of 128
                                 when set.  0 = chosen from the graph: about two
@@ -418,7 +418,7 @@ mm_status mm_skipper_to_host(mm_graph *g, const mm_options *o, uint32_t *d_mate,
  * span graphs).  With local ids or warps_per_graph > 0, every graph is split
  * on its own into min(warps_per_graph, ceil(items / grain)) units (no cap when
  * 0); those tables are computed on the device from d_vbase / d_ebase at every
- * call.  With o->serial each graph is walked by one thread in SGMM order (the
+ * call.  With o->serial each graph is walked by one warp in SGMM order (the
  * result equals sequential greedy MM on every graph).  With o->use_graph the
  * launches run as a CUDA graph built once per handle and option set, whose
  * kernel arguments are updated per call (new buffers or contents need no new
@@ -529,7 +529,7 @@ mm_status mm_autotune_batched(mm_graph *g, uint64_t num_graphs, const int64_t *d
  * pool, checker counters and control words; it grows them (cudaMalloc) only
  * when a call needs more than any earlier call.  Calls on one handle must be
  * ordered (one stream, or synchronised by the caller).
- * mm_skipper_multi: options as mm_skipper (status_bits, serial -- one thread
+ * mm_skipper_multi: options as mm_skipper (status_bits, serial -- one warp
  * per graph in SGMM order --, grain, block_threads, blocks_per_sm, spin_limit,
  * nosync); timing, use_graph, poison_vertex and l2_persist give
  * MM_ERR_UNSUPPORTED.  Waits for the GPU unless nosync (then mm_multi_sync).

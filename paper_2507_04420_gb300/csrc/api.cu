@@ -825,8 +825,8 @@ mm_status build_batch_graph(mm_graph* g, const Resolved& r, uint64_t num_graphs,
   cudaKernelNodeParams ks{};
   ks.func = const_cast<void*>(k_sweep);
   if (r.serial) {
-    ks.gridDim = dim3((unsigned)((num_graphs + 127) / 128));
-    ks.blockDim = dim3(128);
+    ks.gridDim = dim3((unsigned)((num_graphs + kSerialGraphsPerBlock - 1) / kSerialGraphsPerBlock));
+    ks.blockDim = dim3(32 * kSerialGraphsPerBlock);
   } else {
     ks.gridDim = dim3(sweep_grid(g, r, P.lean != 0));
     ks.blockDim = dim3(r.block);
@@ -979,8 +979,8 @@ BatchLaunch batch_launch(const mm_graph* g, const Resolved& r, uint64_t num_grap
   L.prep_grid = dim3(prepare_grid(g));
   L.prep_block = dim3(256);
   if (r.serial) {
-    L.sweep_grid = dim3((unsigned)((num_graphs + 127) / 128));
-    L.sweep_block = dim3(128);
+    L.sweep_grid = dim3((unsigned)((num_graphs + kSerialGraphsPerBlock - 1) / kSerialGraphsPerBlock));
+    L.sweep_block = dim3(32 * kSerialGraphsPerBlock);
   } else {
     const int per_sm = r.blocks_per_sm > 0 ? r.blocks_per_sm
                                            : batch_sweep_blocks_per_sm(r.bits, g->local_ids, r.sym, lean, r.block);

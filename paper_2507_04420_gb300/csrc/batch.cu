@@ -221,18 +221,18 @@ __global__ void __launch_bounds__(512, kLean ? 4 : 3) batch_sweep_kernel(BatchPa
   }
 }
 
-// One thread per graph, rows in ascending order, neighbours in stored order:
+// One warp per graph, rows in ascending order, neighbours in stored order:
 // sequential greedy MM on every graph (Section II-B).
 template <class S, bool kLocal>
 __global__ void batch_serial_kernel(BatchParams B) {
   constexpr bool kWord = S::kPerWord == 1;
-  const uint64_t g = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const uint64_t g = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (g >= B.num_graphs) return;
   const SweepParams P = graph_view<kLocal, kWord>(B, g);
   if (kLocal)
-    serial_rows(S(P), P, 0, P.n);
+    serial_rows(S(P), P, 0, P.n, threadIdx.x & 31u);
   else
-    serial_rows(S(P), P, (uint64_t)B.vbase[g], (uint64_t)B.vbase[g + 1]);
+    serial_rows(S(P), P, (uint64_t)B.vbase[g], (uint64_t)B.vbase[g + 1], threadIdx.x & 31u);
 }
 
 // Matched pairs per graph: vertex i of the batch, in graph g, counts when it

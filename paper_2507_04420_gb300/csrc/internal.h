@@ -19,6 +19,7 @@ bool sweep_lean(int bits, int block_threads, int blocks_per_sm, bool state_fits_
 cudaError_t launch_prepare(const SweepParams& P, int bits, int grid, cudaStream_t s,
                            uint64_t* graph_pairs_zero, uint64_t num_graphs);
 cudaError_t launch_sweep(const SweepParams& P, int bits, int grid, int block, cudaStream_t s);
+constexpr uint64_t kSerialGraphsPerBlock = 4;  // serial batches: one warp walks one graph
 cudaError_t launch_serial(const SweepParams& P, int bits, cudaStream_t s);
 cudaError_t launch_serial_batched(const SweepParams& P, int bits, cudaStream_t s);
 void get_batched_kernels(int bits, bool serial, bool sym, bool lean, const void** prepare,
@@ -46,7 +47,7 @@ struct BatchParams {
 struct BatchKernels {
   const void* plan;        // <<<1, batch_plan_threads()>>>(BatchParams)
   const void* prepare;     // (BatchParams, int states)
-  const void* sweep;       // (BatchParams); the serial kernel takes one thread per graph
+  const void* sweep;       // (BatchParams); the serial kernel takes one warp per graph
   const void* pairs;       // (BatchParams)
 };
 void get_batch_kernels(int bits, bool local, bool serial, bool sym, bool lean, BatchKernels* k);

@@ -128,10 +128,10 @@ __global__ void __launch_bounds__(512, 3) multi_sweep_kernel(MultiParams M) {
 
 template <class S, bool kWord>
 __global__ void multi_serial_kernel(MultiParams M) {
-  const uint64_t g = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const uint64_t g = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;  // one warp a graph
   if (g >= M.num_graphs) return;
   const SweepParams P = view(M, g, kWord);
-  serial_rows(S(P), P, 0, P.n);
+  serial_rows(S(P), P, 0, P.n, threadIdx.x & 31u);
 }
 
 enum { C_MATCHED = 0, C_PAIRS, C_RANGE, C_ASYM, C_NONEDGE, C_UNCOVERED, C_PAIRS_BAD, C_FIRST_BAD,
@@ -490,10 +490,11 @@ mm_status mm_skipper_multi(mm_multi* m, uint64_t num_graphs, const mm_graph_desc
   else multi_prepare_kernel<false><<<prep_grid, 256, 0, s>>>(M);
   MTRY(cudaGetLastError());
   if (o->serial) {
-    const unsigned grid = (unsigned)((num_graphs + 127) / 128);
-    if (bits == 32) multi_serial_kernel<WordState, true><<<grid, 128, 0, s>>>(M);
-    else if (bits == 2) multi_serial_kernel<TwoBitState, false><<<grid, 128, 0, s>>>(M);
-    else multi_serial_kernel<ByteState, false><<<grid, 128, 0, s>>>(M);
+    const unsigned grid = (unsigned)((num_graphs + kSerialGraphsPerBlock - 1) / kSerialGraphsPerBlock);
+    constexpr int threads = 32 * (int)kSerialGraphsPerBlock;
+    if (bits == 32) multi_serial_kernel<WordState, true><<<grid, threads, 0, s>>>(M);
+    else if (bits == 2) multi_serial_kernel<TwoBitState, false><<<grid, threads, 0, s>>>(M);
+    else multi_serial_kernel<ByteState, false><<<grid, threads, 0, s>>>(M);
   } else if (L.units) {
     int per_sm = (int)o->blocks_per_sm;
     if (per_sm <= 0) {

@@ -227,6 +227,17 @@ struct PackedState {
   __device__ static __forceinline__ bool matched(uint32_t raw, uint32_t v) {
     return ((raw >> shift(v)) & kMask) == kMchd;
   }
+  __device__ static __forceinline__ bool reserved(uint32_t raw, uint32_t v) {
+    return ((raw >> shift(v)) & kMask) == kRsvd;
+  }
+  // (u, v) matched by the only warp that touches their two fields (both ACC);
+  // neighbouring fields of the words may belong to another warp's graph
+  __device__ __forceinline__ void match_alone(uint32_t u, uint32_t v) const {
+    mate[u] = v;
+    mate[v] = u;
+    atomicOr(words + word(u), kMchd << shift(u));
+    atomicOr(words + word(v), kMchd << shift(v));
+  }
   // CAS of v's field from `expect` to `desired` starting at the observed word
   // `cur`; a failure caused only by a neighbouring field is retried (it is not
   // a conflict on v).  On failure `cur` holds the word whose field for v is not
@@ -298,6 +309,11 @@ struct WordState {
   __device__ __forceinline__ uint32_t raw(uint32_t v) const { return ld_relaxed(words + v); }
   __device__ __forceinline__ uint32_t peek(uint32_t v) const { return ld_relaxed_nf(words + v); }
   __device__ static __forceinline__ bool matched(uint32_t raw, uint32_t) { return raw < kWRsvd; }
+  __device__ static __forceinline__ bool reserved(uint32_t raw, uint32_t) { return raw == kWRsvd; }
+  __device__ __forceinline__ void match_alone(uint32_t u, uint32_t v) const {
+    st_relaxed(words + u, v);
+    st_relaxed(words + v, u);
+  }
   __device__ __forceinline__ bool try_reserve(uint32_t u, uint32_t& ru, const SweepParams&) const {
     ru = atomicCAS(words + u, kWAcc, kWRsvd);
     return ru == kWAcc;

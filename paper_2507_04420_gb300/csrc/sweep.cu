@@ -13,8 +13,8 @@
 //   rows skipped without a load, unmatched entries read 128 at a time with
 //   128-bit loads, filtered by the states of both endpoints, and the surviving
 //   candidates of one row tried one lane at a time.
-// serial kernels: one thread, rows in ascending order, neighbours in stored
-//   order -- the sequential greedy order (Section II-B).
+// serial kernels: one warp (a graph), rows in ascending order, neighbours in
+//   stored order -- the sequential greedy order (Section II-B).
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -114,16 +114,16 @@ __global__ void __launch_bounds__(512, kLean ? 4 : 3) sweep_kernel(SweepParams P
 
 template <class S>
 __global__ void serial_kernel(SweepParams P) {
-  if (blockIdx.x == 0 && threadIdx.x == 0) serial_rows(S(P), P, 0, P.n);
+  serial_rows(S(P), P, 0, P.n, threadIdx.x);  // one warp
 }
 
 template <class S>
 __global__ void serial_batched_kernel(SweepParams P) {
-  const uint64_t g = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const uint64_t g = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (g < P.num_graphs) {
     uint64_t r0 = (uint64_t)P.vbase[g], r1 = (uint64_t)P.vbase[g + 1];
     r1 = r1 < P.n ? r1 : P.n;  // rows past n do not exist
-    if (r0 < r1) serial_rows(S(P), P, r0, r1);
+    if (r0 < r1) serial_rows(S(P), P, r0, r1, threadIdx.x & 31u);
   }
 }
 
@@ -229,16 +229,16 @@ cudaError_t launch_sweep(const SweepParams& P, int bits, int grid, int block, cu
 }
 
 cudaError_t launch_serial(const SweepParams& P, int bits, cudaStream_t s) {
-#define L(S, B) (serial_kernel<S><<<1, 1, 0, s>>>(P), 0)
+#define L(S, B) (serial_kernel<S><<<1, 32, 0, s>>>(P), 0)
   SKP_DISPATCH_STATE(bits, L);
 #undef L
   return cudaGetLastError();
 }
 
 cudaError_t launch_serial_batched(const SweepParams& P, int bits, cudaStream_t s) {
-  const unsigned grid = (unsigned)((P.num_graphs + 127) / 128);
+  const unsigned grid = (unsigned)((P.num_graphs + kSerialGraphsPerBlock - 1) / kSerialGraphsPerBlock);
   if (grid == 0) return cudaSuccess;
-#define L(S, B) (serial_batched_kernel<S><<<grid, 128, 0, s>>>(P), 0)
+#define L(S, B) (serial_batched_kernel<S><<<grid, 32 * kSerialGraphsPerBlock, 0, s>>>(P), 0)
   SKP_DISPATCH_STATE(bits, L);
 #undef L
   return cudaGetLastError();

@@ -13,8 +13,9 @@ namespace skp {
 namespace {
 
 // a[j] for a run-time j without local-memory indexing
-__device__ __forceinline__ uint32_t pick4(const uint32_t (&a)[4], int j) {
-  uint32_t r = a[0];
+template <class T>
+__device__ __forceinline__ T pick4(const T (&a)[4], int j) {
+  T r = a[0];
 #pragma unroll
   for (int i = 1; i < 4; ++i) r = j == i ? a[i] : r;
   return r;
@@ -326,20 +327,127 @@ __device__ __forceinline__ void sweep_unit(const S& s, const SweepParams& P, int
   }
 }
 
+// Rows [r0, r1) in sequential greedy order (Section II-B: rows ascending,
+// neighbours in stored order, the first free one taken), walked by one warp
+// that is the only one to touch these vertices' states.
+//
+// Greedy order is a chain of decisions, bound by latency: one thread paid two
+// dependent memory round trips for every entry.  Here the warp reads a window
+// of 32 rows and then up to 128 entries at a time -- the ids one chunk ahead,
+// the window's row states beside the first chunk's -- so a chunk costs one
+// round trip, for the states of its vertices, and its decisions are made in
+// registers: the first entry, in stored order, whose two vertices are both
+// free is a pair, and every entry of the chunk that names either is dropped.
+// A call on 4096 graphs of 100 to 10,000 edges (22 M entries, byte states):
+// 16.5 ms with one thread a graph, 0.88 ms with one warp; one Erdos-Renyi
+// graph of 2 M entries 330 -> 28 ms.
 template <class S>
 __device__ __forceinline__ void serial_rows(const S& s, const SweepParams& P, uint64_t r0,
-                                            uint64_t r1) {
-  for (uint64_t x = r0; x < r1; ++x) {
-    if (S::matched(s.raw((uint32_t)x), (uint32_t)x)) continue;
-    for (int64_t i = P.offsets[x]; i < P.offsets[x + 1]; ++i) {
-      const uint32_t y = P.nbrs[i];
-      if (y >= P.n) {
-        atomicOr(P.err, kErrBadId);
-        continue;
+                                            uint64_t r1, const unsigned lane) {
+  const uint64_t pol = policy_evict_first();
+  const uint32_t n32 = (uint32_t)P.n;
+  uint32_t next[4] = {0u, 0u, 0u, 0u};  // ids at next_at + 4 * lane
+  int64_t next_at = -256;
+  int64_t begin = 0, end = 0;           // row ends of the window after this one
+  if (r0 + lane < r1) {
+    begin = __ldg(P.offsets + r0 + lane);
+    end = __ldg(P.offsets + r0 + lane + 1);
+  }
+  for (uint64_t wb = r0; wb < r1; wb += 32) {
+    const bool in = wb + lane < r1;
+    const int64_t my_begin = begin, my_end = end;
+    if (wb + 32 + lane < r1) {
+      begin = __ldg(P.offsets + wb + 32 + lane);
+      end = __ldg(P.offsets + wb + 32 + lane + 1);
+    }
+    // the row states arrive beside the first chunk's: until then every row reads as open
+    const uint32_t my_st = in ? s.raw((uint32_t)(wb + lane)) : 0u;
+    unsigned done = __ballot_sync(kFull, !in);  // vertices of the window that are matched (or past the last row)
+    bool fresh = true;
+    const int rows = r1 - wb < 32 ? (int)(r1 - wb) : 32;
+    const int64_t win_end = __shfl_sync(kFull, my_end, rows - 1);
+    const uint32_t wb32 = (uint32_t)wb;
+    int64_t pos = 0;
+    for (;;) {
+      const unsigned open = __ballot_sync(kFull, my_end > pos) & ~done;
+      if (open == 0u) break;
+      const int64_t st = __shfl_sync(kFull, my_begin, __ffs(open) - 1);
+      if (st > pos) pos = st;
+      if (pos >= win_end) break;  // only empty rows were left
+      const bool loaded = pos >= next_at && pos < next_at + 128;
+      const int64_t base = loaded ? next_at : pos & ~(int64_t)3;
+      const int64_t cend = base + 128 < win_end ? base + 128 : win_end;
+      const int lo_r = (int)(pos - base), hi_r = (int)(cend - base), p0 = 4 * (int)lane;
+      uint32_t y[4] = {next[0], next[1], next[2], next[3]};
+      if (!loaded && p0 < hi_r) load_quad(P, base + p0, pol, y);
+      next_at = base + 128 <= win_end ? base + 128 : win_end & ~(int64_t)3;
+      load_quad(P, next_at + p0, pol, next);
+      const int64_t d = my_end - base;
+      const int rel = lane >= (unsigned)rows || d > 129 ? 129 : d < 0 ? -1 : (int)d;
+      int k[4];
+      uint32_t ry[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) k[j] = count_le(rel, p0 + j) & 31;
+      uint32_t cand = 0;  // entries of open rows, loops apart; an id out of range stays, to be reported in its turn
+      uint32_t bits[4];   // the window's rows that an entry names: its own, and y's if y is one of them
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int p = p0 + j;
+        bits[j] = 1u << k[j] | (y[j] < n32 && y[j] - wb32 < 32u ? 1u << (y[j] - wb32) : 0u);
+        if (p < lo_r || p >= hi_r || (done >> k[j] & 1u) || y[j] == wb32 + (uint32_t)k[j]) continue;
+        cand |= 1u << j;
+        if (y[j] < n32) ry[j] = s.raw(y[j]);
       }
-      if (y == x) continue;
-      if (resolve_edge(s, (uint32_t)x, y, s.raw((uint32_t)x), s.raw(y), P)) break;
-      if (ld_relaxed(P.err) & kErrTimeout) return;
+      if (fresh) {
+        done |= __ballot_sync(kFull, in && S::matched(my_st, wb32 + lane));
+        fresh = false;
+      }
+      bool odd = in && S::reserved(my_st, wb32 + lane);  // entries that take the slow way below
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if ((bits[j] & done) || (y[j] < n32 && S::matched(ry[j], y[j]))) cand &= ~(1u << j);
+        odd |= (cand >> j & 1u) && (y[j] >= n32 || S::reserved(ry[j], y[j]));
+      }
+      const bool any_odd = __any_sync(kFull, odd);
+      uint32_t sx = 0, sy = 0;  // the chunk's i-th pair, on lane i
+      int pairs = 0;
+      for (;;) {
+        const unsigned have = __ballot_sync(kFull, cand != 0u);
+        if (have == 0u) break;
+        const int first = __ffs(have) - 1;
+        const int j = __ffs(cand) - 1;  // -1, and pick4's first, on the lanes without one
+        const uint32_t yv = __shfl_sync(kFull, pick4(y, j), first);
+        const int kx = __shfl_sync(kFull, pick4(k, j), first);
+        const uint32_t xv = wb32 + (uint32_t)kx;
+        if (any_odd) {  // an id out of range, or a poisoned vertex: wait for it, as any thread would
+          uint32_t got = 0;
+          if ((int)lane == first) {
+            cand &= cand - 1u;
+            if (yv >= n32) {
+              atomicOr(P.err, kErrBadId);
+            } else {
+              got = resolve_edge(s, xv, yv, s.raw(xv), s.raw(yv), P) ? 1u : 0u;
+              got |= ld_relaxed(P.err) & kErrTimeout ? 2u : 0u;
+            }
+          }
+          got = __shfl_sync(kFull, got, first);
+          if (got & 2u) return;
+          if (!(got & 1u)) continue;
+        } else {
+          if ((int)lane == pairs) {
+            sx = xv;
+            sy = yv;
+          }
+          ++pairs;  // at most one a row of the window
+        }
+        done |= 1u << kx | (yv - wb32 < 32u ? 1u << (yv - wb32) : 0u);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if ((bits[i] & done) || y[i] == yv) cand &= ~(1u << i);
+      }
+      if ((int)lane < pairs) s.match_alone(sx, sy);
+      __syncwarp();  // the chunk's states are written before the next reads
+      pos = cend;
     }
   }
 }
