@@ -77,14 +77,15 @@ struct mm_graph {
   int64_t* part = nullptr;
   uint64_t part_units_cap = 0;
   unsigned long long* ctrl = nullptr;  // [0] work counter, [1] err word, [2] csr-check count,
-                                       // [8..16] checker counters
+                                       // [8..18] checker counters, zero between checks;
+                                       // [20..23] census
   uint32_t* seen_bits = nullptr;
   unsigned long long* stats = nullptr;  // sweep statistics, allocated on first stats call
   bool stats_valid = false;
   int last_bits = 0;                   // layout and state array of the last mm_skipper call
   const uint32_t* last_state = nullptr;
   unsigned char* found = nullptr;      // checker scratch, allocated on first mm_validate
-  int64_t* check_part = nullptr;
+  uint64_t* long_rows = nullptr;
   uint64_t* tile_counts = nullptr;
   uint64_t tile_cap = 0;
   uint32_t* h_err = nullptr;           // pinned
@@ -122,6 +123,11 @@ unsigned long long* work_ptr(mm_graph* g) { return g->ctrl; }
 uint32_t* err_ptr(mm_graph* g) { return reinterpret_cast<uint32_t*>(g->ctrl + 1); }
 unsigned long long* csr_bad_ptr(mm_graph* g) { return g->ctrl + 2; }
 unsigned long long* counters_ptr(mm_graph* g) { return g->ctrl + 8; }
+unsigned long long* census_ptr(mm_graph* g) { return g->ctrl + 20; }
+
+CheckScratch check_scratch(mm_graph* g) {
+  return CheckScratch{counters_ptr(g), g->h_counters, g->seen_bits, g->tile_counts, g->tile_cap, g->found, g->long_rows};
+}
 
 struct Resolved {
   int bits;   // state layout: 2, 8 (packed fields) or 32 (word = mate)
@@ -477,7 +483,7 @@ mm_status skipper_coo(mm_graph* g, const Resolved& r, uint32_t* d_mate, uint32_t
     C.P.stats = g->stats;
     g->stats_valid = true;
   }
-  CheckScratch cs{counters_ptr(g), g->seen_bits, g->tile_counts, g->tile_cap, nullptr, nullptr};
+  CheckScratch cs = check_scratch(g);
   g->last_bits = r.bits;
   g->last_state = C.P.state;
   cudaEvent_t* ev = nullptr;
@@ -640,7 +646,7 @@ mm_status mm_skipper(mm_graph* g, const mm_options* o, uint32_t* d_mate, uint32_
     g->stats_valid = true;
   }
 
-  CheckScratch cs{counters_ptr(g), g->seen_bits, g->tile_counts, g->tile_cap, nullptr, nullptr};
+  CheckScratch cs = check_scratch(g);
   g->last_bits = r.bits;
   g->last_state = P.state;
   cudaEvent_t* ev = nullptr;
@@ -768,7 +774,7 @@ mm_status mm_state_census(mm_graph* g, uint64_t out[4], void* cuda_stream) {
   if (!out) return fail(MM_ERR_ARG, "null out");
   if (!g->last_state && g->n) return fail(MM_ERR_ARG, "no mm_skipper call on this handle");
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-  unsigned long long* d = counters_ptr(g);  // the checker's counters, free between calls
+  unsigned long long* d = census_ptr(g);
   CUDA_TRY(launch_census(g->last_state, g->n, g->last_bits ? g->last_bits : 8, d, prepare_grid(g), s));
   CUDA_TRY(cudaMemcpyAsync(g->h_counters, d, 4 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
   CUDA_TRY(cudaStreamSynchronize(s));
@@ -1000,9 +1006,7 @@ mm_status build_batch_graph2(mm_graph* g, const Resolved& r, uint64_t num_graphs
   b = BatchGraph{};
   const BatchLaunch L = batch_launch(g, r, num_graphs);
   CUDA_TRY(cudaGraphCreate(&b.graph, 0));
-  int states = 1;
   void* a1[] = {&B};
-  void* a2[] = {&B, &states};
   cudaKernelNodeParams kp{};
   kp.func = const_cast<void*>(L.k.plan);
   kp.gridDim = L.plan_grid;
@@ -1012,7 +1016,7 @@ mm_status build_batch_graph2(mm_graph* g, const Resolved& r, uint64_t num_graphs
   kp.func = const_cast<void*>(L.k.prepare);
   kp.gridDim = L.prep_grid;
   kp.blockDim = L.prep_block;
-  kp.kernelParams = a2;
+  kp.kernelParams = a1;
   CUDA_TRY(cudaGraphAddKernelNode(&b.n_prepare, b.graph, &b.n_plan, 1, &kp));
   kp.func = const_cast<void*>(L.k.sweep);
   kp.gridDim = L.sweep_grid;
@@ -1047,15 +1051,13 @@ mm_status build_batch_graph2(mm_graph* g, const Resolved& r, uint64_t num_graphs
 // New arguments (buffers, tables) for the kernel nodes of the built graph.
 mm_status update_batch_graph2(mm_graph* g, BatchParams B) {
   BatchGraph& b = g->bg2;
-  int states = 1;
   void* a1[] = {&B};
-  void* a2[] = {&B, &states};
   cudaGraphNode_t nodes[] = {b.n_plan, b.n_prepare, b.n_sweep, b.n_pairs};
   for (int i = 0; i < 4; ++i) {
     if (!nodes[i]) continue;
     cudaKernelNodeParams kp{};
     CUDA_TRY(cudaGraphKernelNodeGetParams(nodes[i], &kp));
-    kp.kernelParams = i == 1 ? a2 : a1;
+    kp.kernelParams = a1;
     kp.extra = nullptr;
     CUDA_TRY(cudaGraphExecKernelNodeSetParams(b.exec, nodes[i], &kp));
   }
@@ -1092,11 +1094,9 @@ mm_status run_batched2(mm_graph* g, const Resolved& r, uint64_t num_graphs, cons
     ev = next_hist(g, 0, d_graph_pairs != nullptr);
     CUDA_TRY(cudaEventRecord(ev[0], s));
   }
-  int states = 1;
   void* a1[] = {&B};
-  void* a2[] = {&B, &states};
   CUDA_TRY(cudaLaunchKernel(L.k.plan, L.plan_grid, L.plan_block, a1, 0, s));
-  CUDA_TRY(cudaLaunchKernel(L.k.prepare, L.prep_grid, L.prep_block, a2, 0, s));
+  CUDA_TRY(cudaLaunchKernel(L.k.prepare, L.prep_grid, L.prep_block, a1, 0, s));
   if (ev) CUDA_TRY(cudaEventRecord(ev[1], s));
   CUDA_TRY(cudaLaunchKernel(L.k.sweep, L.sweep_grid, L.sweep_block, a1, 0, s));
   if (ev) CUDA_TRY(cudaEventRecord(ev[2], s));
@@ -1175,6 +1175,12 @@ mm_status mm_skipper_batched(mm_graph* g, uint64_t num_graphs, const int64_t* d_
   return read_err(g, s);
 }
 
+static mm_status ensure_long_rows(mm_graph* g) {
+  const uint64_t cap = long_row_cap(g->nnz);
+  if (cap && !g->long_rows) CUDA_TRY(cudaMalloc(&g->long_rows, cap * sizeof(uint64_t)));
+  return MM_OK;
+}
+
 mm_status mm_validate(mm_graph* g, const uint32_t* d_mate, const uint32_t* d_pairs, uint64_t count,
                       mm_verdict* h_out, void* cuda_stream) {
   g_err[0] = 0;
@@ -1188,18 +1194,13 @@ mm_status mm_validate(mm_graph* g, const uint32_t* d_mate, const uint32_t* d_pai
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   if (g->coo) {
     if (!g->found) CUDA_TRY(cudaMalloc(&g->found, g->n + 16));
-    CheckScratch cs{counters_ptr(g), g->seen_bits, g->tile_counts, g->tile_cap, g->found, nullptr};
-    CUDA_TRY(launch_validate_coo(g->n, g->nnz, g->src, g->dst, d_mate, d_pairs, d_pairs ? count : 0, cs,
-                                 prepare_grid(g), s));
+    CUDA_TRY(launch_validate_coo(g->n, g->nnz, g->src, g->dst, d_mate, d_pairs, d_pairs ? count : 0,
+                                 check_scratch(g), g->num_sms, s));
   } else {
-    if (!g->check_part)
-      CUDA_TRY(cudaMalloc(&g->check_part, ((g->n + g->nnz) / kCheckGrain + 2) * 2 * sizeof(int64_t)));
-    CheckScratch cs{counters_ptr(g), g->seen_bits, g->tile_counts, g->tile_cap, nullptr, g->check_part};
-    CUDA_TRY(launch_validate(g->n, g->nnz, g->offsets, g->nbrs, d_mate, d_pairs, d_pairs ? count : 0, cs,
-                             prepare_grid(g), s));
+    if ((st = ensure_long_rows(g)) != MM_OK) return st;
+    CUDA_TRY(launch_validate(g->n, g->nnz, g->offsets, g->nbrs, d_mate, d_pairs, d_pairs ? count : 0,
+                             check_scratch(g), g->num_sms, s));
   }
-  CUDA_TRY(cudaMemcpyAsync(g->h_counters, counters_ptr(g), 9 * sizeof(unsigned long long),
-                           cudaMemcpyDeviceToHost, s));
   CUDA_TRY(cudaStreamSynchronize(s));
   const unsigned long long* c = g->h_counters;
   mm_verdict v{};
@@ -1232,16 +1233,22 @@ mm_status mm_validate_batched(mm_graph* g, uint64_t num_graphs, const int64_t* d
   if (num_graphs == 0 || num_graphs >= (1ull << 32)) return fail(MM_ERR_ARG, "num_graphs must be in [1, 2^32)");
   if (!d_vbase || !d_ebase) return fail(MM_ERR_ARG, "null vbase / ebase");
   if (!d_mate && g->n) return fail(MM_ERR_ARG, "null mate");
-  if ((st = ensure_batch_scratch(g, num_graphs, kCheckGrain, 32)) != MM_OK) return st;
-  Resolved r{};
-  r.grain = (uint32_t)kCheckGrain;
-  r.bits = 32;
-  r.word = true;
-  const BatchParams B = batch_params(g, r, num_graphs, d_vbase, d_ebase, const_cast<uint32_t*>(d_mate), nullptr);
+  if ((st = ensure_long_rows(g)) != MM_OK) return st;
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-  CUDA_TRY(launch_validate_batch(B, counters_ptr(g), prepare_grid(g), s));
-  CUDA_TRY(cudaMemcpyAsync(g->h_counters, counters_ptr(g), 9 * sizeof(unsigned long long),
-                           cudaMemcpyDeviceToHost, s));
+  if (g->local_ids) {
+    BatchParams B{};
+    B.P.n = g->n;
+    B.P.nnz = g->nnz;
+    B.P.offsets = g->offsets;
+    B.P.nbrs = g->nbrs;
+    B.P.mate = const_cast<uint32_t*>(d_mate);
+    B.vbase = d_vbase;
+    B.num_graphs = num_graphs;
+    CUDA_TRY(launch_validate_batch(B, check_scratch(g), g->num_sms, s));
+  } else {  // no entry leaves its graph: the batch is checked as one CSR
+    CUDA_TRY(launch_validate(g->n, g->nnz, g->offsets, g->nbrs, d_mate, nullptr, 0, check_scratch(g),
+                             g->num_sms, s));
+  }
   CUDA_TRY(cudaStreamSynchronize(s));
   const unsigned long long* c = g->h_counters;
   mm_verdict v{};
@@ -1409,7 +1416,7 @@ mm_status mm_destroy(mm_graph* g) {
   if (g->seen_bits) cudaFree(g->seen_bits);
   if (g->found) cudaFree(g->found);
   if (g->stats) cudaFree(g->stats);
-  if (g->check_part) cudaFree(g->check_part);
+  if (g->long_rows) cudaFree(g->long_rows);
   if (g->tile_counts) cudaFree(g->tile_counts);
   if (g->h_err) cudaFreeHost(g->h_err);
   if (g->h_counters) cudaFreeHost(g->h_counters);

@@ -153,21 +153,18 @@ __device__ __forceinline__ void fill(uint32_t* p, uint64_t count, uint32_t value
 }
 
 // Algorithm 1 lines 3-4 (every vertex ACC, mate unmatched) and the merge-path
-// units of every graph (after batch_plan_kernel).  With `states` false only
-// the units are made (the checker's partition).
+// units of every graph (after batch_plan_kernel).
 template <int kBits>
-__global__ void batch_prepare_kernel(BatchParams B, int states) {
+__global__ void batch_prepare_kernel(BatchParams B) {
   const uint64_t tid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const uint64_t nthreads = (uint64_t)gridDim.x * blockDim.x;
   const uint64_t n = B.P.n;
   const uint64_t G = B.num_graphs;
-  if (states) {
-    if (kBits == 32) {
-      fill(B.P.mate, n, kWAcc, tid, nthreads);
-    } else {
-      fill(B.P.state, B.local ? B.totals[1] : packed_words(n, kBits), 0u, tid, nthreads);
-      fill(B.P.mate, n, kNone, tid, nthreads);
-    }
+  if (kBits == 32) {
+    fill(B.P.mate, n, kWAcc, tid, nthreads);
+  } else {
+    fill(B.P.state, B.local ? B.totals[1] : packed_words(n, kBits), 0u, tid, nthreads);
+    fill(B.P.mate, n, kNone, tid, nthreads);
   }
   const uint64_t units = B.totals[0];
   for (uint64_t u = tid; u < units; u += nthreads) {
@@ -184,12 +181,10 @@ __global__ void batch_prepare_kernel(BatchParams B, int states) {
     B.part[2 * u + 1] = eb + d - rows;
     B.gid[u] = (uint32_t)g;
   }
-  if (states) {
-    for (uint64_t g = tid; g < G && B.graph_pairs; g += nthreads) B.graph_pairs[g] = 0;
-    if (tid == 0) {
-      *B.P.work = 0ull;
-      *B.P.err = 0u;
-    }
+  for (uint64_t g = tid; g < G && B.graph_pairs; g += nthreads) B.graph_pairs[g] = 0;
+  if (tid == 0) {
+    *B.P.work = 0ull;
+    *B.P.err = 0u;
   }
 }
 
@@ -262,111 +257,52 @@ __global__ void batch_pairs_kernel(BatchParams B) {
   }
 }
 
-// ---- the exact checker over a batch (Section II-B), one verdict for all
-// member graphs; vertex and entry indices are the batch's (global) ones ----
-enum { BC_MATCHED = 0, BC_PAIRS, BC_RANGE, BC_ASYM, BC_NONEDGE, BC_UNCOVERED, BC_PAIRS_BAD,
-       BC_FIRST_BAD, BC_FIRST_UNCOVERED, BC_N };
+// ---- the exact checker over a batch of graphs with local ids (Section II-B),
+// one verdict for all member graphs; the vertex and entry indices it names are
+// the batch's.  (With global ids a batch is one CSR: launch_validate.)  A warp
+// takes runs of kCheckRun * 32 vertices, so that one search of vbase serves a
+// run and a lane then only steps on to the next graph. ----
+constexpr uint64_t kCheckRun = 8;
 
-__global__ void batch_check_init_kernel(unsigned long long* c) {
-  if (threadIdx.x < BC_N) c[threadIdx.x] = threadIdx.x >= BC_FIRST_BAD ? ~0ull : 0ull;
+__device__ __forceinline__ CheckView batch_check_view(const BatchParams& B, uint64_t g) {
+  const int64_t vb = __ldg(B.vbase + g);
+  return CheckView{B.P.offsets + vb, B.P.nbrs, B.P.mate + vb, (uint64_t)(__ldg(B.vbase + g + 1) - vb), B.P.nnz};
 }
 
-// edge pass: the uncovered entries of every unit of every graph
-template <bool kLocal>
-__global__ void batch_check_edges_kernel(BatchParams B, unsigned long long* c) {
-  const unsigned lane = threadIdx.x & 31u;
-  const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-  const uint64_t units = B.totals[0];
-  unsigned long long unc = 0, first = ~0ull;
-  for (uint64_t u = warp; u < units; u += nwarps) {
-    const uint32_t g = B.gid[u];
-    const SweepParams P = graph_view<kLocal, true>(B, g);
-    const int64_t e0 = B.part[2 * u + 1];
-    const int64_t e1 = (u + 1 < units && B.gid[u + 1] == g) ? B.part[2 * u + 3] : B.ebase[g + 1];
-    if (e0 < e1) check_unit(P.offsets, P.nbrs, P.n, P.nnz, P.mate, B.part[2 * u], e0, e1, lane, unc, first);
-  }
-  unc = warp_sum64(unc);
-  first = warp_min64(first);
-  if (lane == 0) {
-    if (unc) atomicAdd(c + BC_UNCOVERED, unc);
-    if (first != ~0ull) atomicMin(c + BC_FIRST_UNCOVERED, first);
-  }
-}
-
-// vertex pass (range, symmetry, pairs) and existence pass (the named partner
-// shares an edge, stored in either row, the shorter row searched first), one
-// warp per 32 consecutive vertices of the batch
-template <bool kLocal>
-__global__ void batch_check_vertices_kernel(BatchParams B, unsigned long long* c) {
+__global__ void __launch_bounds__(256, kCheckBlocks) batch_check_kernel(BatchParams B, LongRows queue,
+                                                             unsigned long long* __restrict__ c,
+                                                             unsigned long long* __restrict__ host) {
   const unsigned lane = threadIdx.x & 31u;
   const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
   const uint64_t N = B.P.n, G = B.num_graphs;
-  unsigned long long matched = 0, pairs = 0, range = 0, asym = 0, nonedge = 0, first_bad = ~0ull;
-  for (uint64_t w0 = warp * 32; w0 < N; w0 += nwarps * 32) {
-    const uint64_t i = w0 + lane;
-    uint64_t g = 0, vb = 0, ng = N;
-    uint32_t v = 0, m = kNone;
-    bool valid = false, sym = false;
-    if (i < N) {
-      if (kLocal) {
-        g = last_at_or_below(B.vbase, G, i);
-        vb = (uint64_t)B.vbase[g];
-        ng = (uint64_t)B.vbase[g + 1] - vb;
-      }
-      v = (uint32_t)(i - vb);
-      m = B.P.mate[i];
-      if (m != kNone) {
-        if (m >= ng || m == v) {
-          ++range;
-          if (i < first_bad) first_bad = i;
-        } else {
-          ++matched;
-          valid = true;
-          sym = B.P.mate[vb + m] == v;
-          if (!sym) {
-            ++asym;
-            if (i < first_bad) first_bad = i;
-          } else if (v < m) {
-            ++pairs;
-          }
-        }
-      }
-    }
-    unsigned todo = __ballot_sync(kFull, valid && !(sym && m < v));
-    while (todo) {
-      const int j = __ffs(todo) - 1;
-      todo &= todo - 1;
-      const uint64_t vbj = __shfl_sync(kFull, vb, j);
-      const uint32_t vj = __shfl_sync(kFull, v, j), mj = __shfl_sync(kFull, m, j);
-      const bool sj = __shfl_sync(kFull, sym ? 1u : 0u, j) != 0u;
-      const int64_t* off = B.P.offsets + (kLocal ? vbj : 0);
-      const int64_t dv = off[vj + 1] - off[vj];
-      const int64_t dm = off[mj + 1] - off[mj];
-      const bool v_first = dv <= dm;  // the shorter row first
-      bool hit = warp_row_has(off, B.P.nbrs, v_first ? vj : mj, v_first ? mj : vj, lane);
-      if (!hit) hit = warp_row_has(off, B.P.nbrs, v_first ? mj : vj, v_first ? vj : mj, lane);
-      if (!hit && lane == 0) {
-        nonedge += sj ? 2 : 1;
-        if (vbj + vj < first_bad) first_bad = vbj + vj;
-      }
+  uint32_t matched = 0, pairs = 0;
+  for (uint64_t w0 = warp * 32 * kCheckRun; w0 < N; w0 += nwarps * 32 * kCheckRun) {
+    uint64_t g = warp_last_at_or_below(B.vbase, G, w0, lane);
+    for (uint64_t v0 = w0; v0 < w0 + 32 * kCheckRun && v0 < N; v0 += 32) {
+      const uint64_t i = v0 + lane;
+      const bool in = i < N;
+      while (in && (int64_t)i >= __ldg(B.vbase + g + 1)) ++g;
+      const CheckView V = batch_check_view(B, g);
+      const uint64_t vb = (uint64_t)(V.mate - B.P.mate);
+      const Visit a = check_group<false>(V, in, (uint32_t)(i - vb), (uint32_t)g, lane, queue);
+      matched += __popc(__ballot_sync(kFull, a.bits & kVxMatched));
+      pairs += __popc(__ballot_sync(kFull, a.bits & kVxPair));
+      add_faults(c, a, i, lane);
     }
   }
-  matched = warp_sum64(matched);
-  pairs = warp_sum64(pairs);
-  range = warp_sum64(range);
-  asym = warp_sum64(asym);
-  nonedge = warp_sum64(nonedge);
-  first_bad = warp_min64(first_bad);
-  if (lane == 0) {
-    if (matched) atomicAdd(c + BC_MATCHED, matched);
-    if (pairs) atomicAdd(c + BC_PAIRS, pairs);
-    if (range) atomicAdd(c + BC_RANGE, range);
-    if (asym) atomicAdd(c + BC_ASYM, asym);
-    if (nonedge) atomicAdd(c + BC_NONEDGE, nonedge);
-    if (first_bad != ~0ull) atomicMin(c + BC_FIRST_BAD, first_bad);
+  add_block(c, matched, pairs);
+  if (host) publish_counters(c, host);
+}
+
+__global__ void batch_check_long_kernel(BatchParams B, LongRows queue, unsigned long long* __restrict__ c,
+                                        unsigned long long* __restrict__ host) {
+  const unsigned long long rows = *queue.count;
+  for (unsigned long long i = 0; i < rows; ++i) {
+    const uint64_t item = queue.items[i];
+    check_long_row(batch_check_view(B, item >> 32), (uint32_t)item, c, threadIdx.x & 31u);
   }
+  publish_counters(c, host);
 }
 
 }  // namespace
@@ -406,23 +342,11 @@ int batch_sweep_blocks_per_sm(int bits, bool local, bool sym, bool lean, int blo
   return b;
 }
 
-// The checker over a batch: partition every graph with the checker's grain
-// (no state is touched), then the edge pass and the vertex pass.
-cudaError_t launch_validate_batch(const BatchParams& B0, unsigned long long* counters, int grid,
-                                  cudaStream_t s) {
-  BatchParams B = B0;
-  B.grain = kCheckGrain;
-  B.wpg = 0;
-  batch_check_init_kernel<<<1, 32, 0, s>>>(counters);
-  batch_plan_kernel<32><<<1, kPlanThreads, 0, s>>>(B);
-  batch_prepare_kernel<32><<<grid, 256, 0, s>>>(B, 0);
-  if (B.local) {
-    batch_check_edges_kernel<true><<<grid, 256, 0, s>>>(B, counters);
-    batch_check_vertices_kernel<true><<<grid, 256, 0, s>>>(B, counters);
-  } else {
-    batch_check_edges_kernel<false><<<grid, 256, 0, s>>>(B, counters);
-    batch_check_vertices_kernel<false><<<grid, 256, 0, s>>>(B, counters);
-  }
+cudaError_t launch_validate_batch(const BatchParams& B, const CheckScratch& cs, int sms, cudaStream_t s) {
+  const LongRows queue{cs.counters + kCkLong, cs.long_rows};
+  const bool has_long = B.P.nnz > (uint64_t)kLongRow;
+  batch_check_kernel<<<check_grid(B.P.n, sms), 256, 0, s>>>(B, queue, cs.counters, has_long ? nullptr : cs.host);
+  if (has_long) batch_check_long_kernel<<<sms * 2, 256, 0, s>>>(B, queue, cs.counters, cs.host);
   return cudaGetLastError();
 }
 

@@ -4,9 +4,9 @@
 // The checker follows the validation rule of Section II-B (every edge touches
 // an output edge; no two output edges share an endpoint) with the counting
 // rules stated in skipper.h, so its verdict can be compared field by field
-// with a host checker.  Counters are aggregated per warp and added with 64-bit
-// atomics; "first offender" fields take the minimum with atomicMin, so every
-// field is independent of thread timing.
+// with a host checker.  Counters are summed per block and added with 64-bit
+// atomics; "first offender" fields take the minimum, so every field is
+// independent of thread timing.
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -17,9 +17,6 @@
 namespace skp {
 
 namespace {
-
-enum { C_MATCHED = 0, C_PAIRS, C_RANGE, C_ASYM, C_NONEDGE, C_UNCOVERED, C_PAIRS_BAD,
-       C_FIRST_BAD, C_FIRST_UNCOVERED, C_COUNT };
 
 __global__ void zero_u64_kernel(unsigned long long* p, uint64_t words, unsigned long long v) {
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < words;
@@ -61,41 +58,36 @@ __device__ __forceinline__ void warp_add(unsigned long long* c, uint32_t v) {
   if ((threadIdx.x & 31) == 0 && s) atomicAdd(c, (unsigned long long)s);
 }
 
-// Merge-path split of rows + entries into units of `grain` items (the same
-// split the sweep uses), for the checker's edge pass.
-__global__ void check_partition_kernel(uint64_t n, uint64_t nnz, const int64_t* __restrict__ offsets,
-                                       uint64_t grain, uint64_t units, int64_t* __restrict__ part) {
-  const int64_t total = (int64_t)(n + nnz);
-  for (uint64_t u = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; u <= units;
-       u += (uint64_t)gridDim.x * blockDim.x) {
-    int64_t d = (int64_t)(u * grain);
-    if (d > total) d = total;
-    const int64_t rows = merge_path_rows(offsets, (int64_t)n, (int64_t)nnz, d);
-    part[2 * u] = rows;
-    part[2 * u + 1] = d - rows;
-  }
-}
-
-// edge pass (checkwalk.cuh): uncovered entries, in the rows of unmatched vertices
-__global__ void validate_edges_kernel(uint64_t n, uint64_t nnz, const int64_t* __restrict__ offsets,
-                                      const uint32_t* __restrict__ nbrs,
-                                      const uint32_t* __restrict__ mate,
-                                      const int64_t* __restrict__ part, uint64_t units,
-                                      unsigned long long* __restrict__ c) {
+// The checker over a CSR (checkwalk.cuh): one warp per 32 consecutive vertices.
+// `host` null: the long rows' kernel runs next and publishes the counters.
+// Both kernels are bound by the latency of dependent reads (four round trips a
+// vertex), so they take the 48 warps an SM that 40 registers leave room for.
+// One visit a vertex replaces a partition, an edge pass, an existence pass with
+// one warp a pair and a vertex pass: CHECK_FIGURES.
+__global__ void __launch_bounds__(256, kCheckBlocks) check_csr_kernel(CheckView V, LongRows queue,
+                                                            unsigned long long* __restrict__ c,
+                                                            unsigned long long* __restrict__ host) {
   const unsigned lane = threadIdx.x & 31u;
   const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-  unsigned long long unc = 0, first = ~0ull;
-  for (uint64_t u = warp; u < units; u += nwarps) {
-    const int64_t e0 = part[2 * u + 1], e1 = part[2 * u + 3];
-    if (e0 < e1) check_unit(offsets, nbrs, n, nnz, mate, part[2 * u], e0, e1, lane, unc, first);
+  uint32_t matched = 0, pairs = 0;
+  for (uint64_t v0 = warp * 32; v0 < V.n; v0 += nwarps * 32) {
+    const Visit a = check_group<true>(V, v0 + lane < V.n, (uint32_t)v0 + lane, 0, lane, queue);
+    matched += __popc(__ballot_sync(kFull, a.bits & kVxMatched));
+    pairs += __popc(__ballot_sync(kFull, a.bits & kVxPair));
+    add_faults(c, a, v0 + lane, lane);
   }
-  unc = warp_sum64(unc);
-  first = warp_min64(first);
-  if (lane == 0) {
-    if (unc) atomicAdd(c + C_UNCOVERED, unc);
-    if (first != ~0ull) atomicMin(c + C_FIRST_UNCOVERED, first);
-  }
+  add_block(c, matched, pairs);
+  if (host) publish_counters(c, host);
+}
+
+// the queued rows of unmatched vertices, each spread over the grid
+__global__ void check_csr_long_kernel(CheckView V, LongRows queue, unsigned long long* __restrict__ c,
+                                      unsigned long long* __restrict__ host) {
+  const unsigned long long rows = *queue.count;
+  for (unsigned long long i = 0; i < rows; ++i)
+    check_long_row(V, (uint32_t)queue.items[i], c, threadIdx.x & 31u);
+  publish_counters(c, host);
 }
 
 // edge pass over an edge list: edge i = (x, y), x != y, both ids < n, is
@@ -127,69 +119,38 @@ __global__ void validate_coo_edges_kernel(uint64_t n, uint64_t m, const uint32_t
   unc = warp_sum64(unc);
   first = warp_min64(first);
   if (lane == 0) {
-    if (unc) atomicAdd(c + C_UNCOVERED, unc);
-    if (first != ~0ull) atomicMin(c + C_FIRST_UNCOVERED, first);
+    if (unc) atomicAdd(c + kCkUncovered, unc);
+    if (~first) atomicMax(c + kCkFirstUncovered, ~first);
   }
 }
 
-// existence pass (checkwalk.cuh): each named partner must share an edge with
-// its vertex; one warp per 32 consecutive vertices
-__global__ void validate_exist_kernel(uint64_t n, const int64_t* __restrict__ offsets,
-                                      const uint32_t* __restrict__ nbrs,
-                                      const uint32_t* __restrict__ mate,
-                                      unsigned long long* __restrict__ c) {
-  const unsigned lane = threadIdx.x & 31u;
-  const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-  unsigned long long nonedge = 0, first = ~0ull;
-  for (uint64_t v0 = warp * 32; v0 < n; v0 += nwarps * 32)
-    check_pairs32(offsets, nbrs, n, mate, v0, lane, nonedge, first);
-  if (lane == 0) {
-    if (nonedge) atomicAdd(c + C_NONEDGE, nonedge);
-    if (first != ~0ull) atomicMin(c + C_FIRST_BAD, first);
-  }
-}
-
-// vertex pass: range / symmetry of each named partner; with `found` (edge
-// lists: the edge pass marks every vertex whose partner edge it met) also its
-// existence -- a CSR's existence pass is validate_exist_kernel
-__global__ void validate_vertex_kernel(uint64_t n, const uint32_t* __restrict__ mate,
-                                       const unsigned char* __restrict__ found,
-                                       unsigned long long* __restrict__ c) {
+// vertex pass of an edge list: range and symmetry of each named partner, and
+// its existence (the edge pass marks every vertex whose partner edge it met)
+__global__ void validate_coo_vertex_kernel(uint64_t n, const uint32_t* __restrict__ mate,
+                                           const unsigned char* __restrict__ found,
+                                           unsigned long long* __restrict__ c,
+                                           unsigned long long* __restrict__ host) {
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+  const unsigned lane = threadIdx.x & 31u;
+  uint32_t matched = 0, pairs = 0;
   for (uint64_t v0 = (uint64_t)blockIdx.x * blockDim.x; v0 < n; v0 += stride) {
     const uint64_t v = v0 + threadIdx.x;
-    uint32_t matched = 0, pair = 0, range = 0, asym = 0, nonedge = 0;
-    bool bad = false;
-    if (v < n) {
-      const uint32_t m = mate[v];
-      if (m != kNone) {
-        if (m >= n || m == v) {
-          range = 1;
-          bad = true;
-        } else {
-          matched = 1;
-          if (mate[m] != (uint32_t)v) {
-            asym = 1;
-            bad = true;
-          } else if (v < m) {
-            pair = 1;
-          }
-          if (found && !found[v] && !found[m]) {  // the edge may be listed either way
-            nonedge = 1;
-            bad = true;
-          }
-        }
+    const uint32_t m = v < n ? mate[v] : kNone;
+    Visit a;
+    if (m != kNone) {
+      if (m >= n || m == v) {
+        a.bits = kVxRange;
+      } else {
+        a.bits = kVxMatched | (mate[m] != (uint32_t)v ? kVxAsym : v < m ? kVxPair : 0u);
+        if (!found[v] && !found[m]) a.bits |= kVxNonedge;  // the edge may be listed either way
       }
     }
-    warp_add(c + C_MATCHED, matched);
-    warp_add(c + C_PAIRS, pair);
-    warp_add(c + C_RANGE, range);
-    warp_add(c + C_ASYM, asym);
-    warp_add(c + C_NONEDGE, nonedge);
-    const uint32_t first_bad = __reduce_min_sync(kFull, bad ? (uint32_t)v : kNone);
-    if ((threadIdx.x & 31) == 0 && first_bad != kNone) atomicMin(c + C_FIRST_BAD, (unsigned long long)first_bad);
+    matched += __popc(__ballot_sync(kFull, a.bits & kVxMatched));
+    pairs += __popc(__ballot_sync(kFull, a.bits & kVxPair));
+    add_faults(c, a, v, lane);
   }
+  add_block(c, matched, pairs);
+  publish_counters(c, host);
 }
 
 __global__ void validate_pairs_kernel(uint64_t n, const uint32_t* __restrict__ mate,
@@ -209,7 +170,7 @@ __global__ void validate_pairs_kernel(uint64_t n, const uint32_t* __restrict__ m
         if (atomicOr(seen + (a >> 5), bit) & bit) bad = 1;  // a repeat of a valid pair
       }
     }
-    warp_add(c + C_PAIRS_BAD, bad);
+    warp_add(c + kCkPairsBad, bad);
   }
 }
 
@@ -315,6 +276,15 @@ __global__ void compact_scatter_kernel(uint64_t n, const uint32_t* __restrict__ 
 
 }  // namespace
 
+// rows of a CSR with nnz entries that can be longer than kLongRow
+uint64_t long_row_cap(uint64_t nnz) { return nnz / (uint64_t)kLongRow; }
+
+// blocks of 256 threads for n vertices: no more than their groups of 32 fill, or than are resident
+int check_grid(uint64_t n, int sms) {
+  const uint64_t blocks = (n + 255) / 256;
+  return blocks < (uint64_t)sms * kCheckBlocks ? (int)(blocks ? blocks : 1) : sms * kCheckBlocks;
+}
+
 cudaError_t launch_csr_check(uint64_t n, uint64_t nnz, const int64_t* offsets,
                              const uint32_t* nbrs, unsigned long long* bad, int grid,
                              cudaStream_t s) {
@@ -325,18 +295,17 @@ cudaError_t launch_csr_check(uint64_t n, uint64_t nnz, const int64_t* offsets,
 
 cudaError_t launch_validate(uint64_t n, uint64_t nnz, const int64_t* offsets, const uint32_t* nbrs,
                             const uint32_t* mate, const uint32_t* pairs, uint64_t count,
-                            const CheckScratch& cs, int grid, cudaStream_t s) {
-  zero_u64_kernel<<<1, 32, 0, s>>>(cs.counters, C_FIRST_BAD, 0ull);
-  zero_u64_kernel<<<1, 32, 0, s>>>(cs.counters + C_FIRST_BAD, 2, ~0ull);
-  if (pairs && count) zero_u32_kernel<<<grid, 256, 0, s>>>(cs.seen_bits, (n + 31) / 32);
-  if (n) {
-    const uint64_t units = (n + nnz + kCheckGrain - 1) / kCheckGrain;
-    check_partition_kernel<<<grid, 256, 0, s>>>(n, nnz, offsets, kCheckGrain, units, cs.part);
-    if (nnz) validate_edges_kernel<<<grid, 256, 0, s>>>(n, nnz, offsets, nbrs, mate, cs.part, units, cs.counters);
-    validate_exist_kernel<<<grid, 256, 0, s>>>(n, offsets, nbrs, mate, cs.counters);
-    validate_vertex_kernel<<<grid, 256, 0, s>>>(n, mate, nullptr, cs.counters);
+                            const CheckScratch& cs, int sms, cudaStream_t s) {
+  const int grid = sms * 8;
+  if (pairs && count) {
+    zero_u32_kernel<<<grid, 256, 0, s>>>(cs.seen_bits, (n + 31) / 32);
+    validate_pairs_kernel<<<grid, 256, 0, s>>>(n, mate, pairs, count, cs.seen_bits, cs.counters);
   }
-  if (pairs && count) validate_pairs_kernel<<<grid, 256, 0, s>>>(n, mate, pairs, count, cs.seen_bits, cs.counters);
+  const CheckView V{offsets, nbrs, mate, n, nnz};
+  const LongRows queue{cs.counters + kCkLong, cs.long_rows};
+  const bool has_long = nnz > (uint64_t)kLongRow;  // else no row is longer
+  check_csr_kernel<<<check_grid(n, sms), 256, 0, s>>>(V, queue, cs.counters, has_long ? nullptr : cs.host);
+  if (has_long) check_csr_long_kernel<<<sms * 2, 256, 0, s>>>(V, queue, cs.counters, cs.host);
   return cudaGetLastError();
 }
 
@@ -349,16 +318,15 @@ cudaError_t launch_coo_check(uint64_t n, uint64_t m, const uint32_t* src, const 
 
 cudaError_t launch_validate_coo(uint64_t n, uint64_t m, const uint32_t* src, const uint32_t* dst,
                                 const uint32_t* mate, const uint32_t* pairs, uint64_t count,
-                                const CheckScratch& cs, int grid, cudaStream_t s) {
-  zero_u64_kernel<<<1, 32, 0, s>>>(cs.counters, C_FIRST_BAD, 0ull);
-  zero_u64_kernel<<<1, 32, 0, s>>>(cs.counters + C_FIRST_BAD, 2, ~0ull);
-  if (pairs && count) zero_u32_kernel<<<grid, 256, 0, s>>>(cs.seen_bits, (n + 31) / 32);
-  if (n) {
-    zero_u32_kernel<<<grid, 256, 0, s>>>(reinterpret_cast<uint32_t*>(cs.found), (n + 3) / 4);
-    if (m) validate_coo_edges_kernel<<<grid, 256, 0, s>>>(n, m, src, dst, mate, cs.found, cs.counters);
-    validate_vertex_kernel<<<grid, 256, 0, s>>>(n, mate, cs.found, cs.counters);
+                                const CheckScratch& cs, int sms, cudaStream_t s) {
+  const int grid = sms * 8;
+  if (pairs && count) {
+    zero_u32_kernel<<<grid, 256, 0, s>>>(cs.seen_bits, (n + 31) / 32);
+    validate_pairs_kernel<<<grid, 256, 0, s>>>(n, mate, pairs, count, cs.seen_bits, cs.counters);
   }
-  if (pairs && count) validate_pairs_kernel<<<grid, 256, 0, s>>>(n, mate, pairs, count, cs.seen_bits, cs.counters);
+  if (n) zero_u32_kernel<<<grid, 256, 0, s>>>(reinterpret_cast<uint32_t*>(cs.found), (n + 3) / 4);
+  if (n && m) validate_coo_edges_kernel<<<grid, 256, 0, s>>>(n, m, src, dst, mate, cs.found, cs.counters);
+  validate_coo_vertex_kernel<<<grid, 256, 0, s>>>(n, mate, cs.found, cs.counters, cs.host);
   return cudaGetLastError();
 }
 

@@ -1,19 +1,24 @@
-// checkwalk.cuh -- the exact checker's two graph passes (Section II-B: every
-// graph edge touches an output edge; each output edge is a graph edge), shared
-// by the single-graph and multi-graph checkers.
+// checkwalk.cuh -- the exact checker's walk (Section II-B: every graph edge
+// touches an output edge; each output edge is a graph edge; no vertex is in
+// two), shared by the single-graph, packed-batch and multi-graph checkers.
 //
-// Edge pass (check_unit), over one merge-path unit: an entry (x, y), x != y,
-// is uncovered when mate[x] and mate[y] are both unmatched -- so only the rows
-// of unmatched vertices can hold one.  The walk keeps 32-row windows (row ends
-// and mates in one step, like the sweep) and leaves every row whose mate is
-// set; the remaining entries are read 128 at a time.
+// One warp takes 32 consecutive vertices, one a lane (check_group), and does
+// all of a vertex's checking in one visit:
+//   v matched to m: m in range, mate[m] == v, and an edge between them, stored
+//     in row v or in row m (the CSR may hold an edge for one endpoint only):
+//     the shorter row is searched first and left at the first hit; a symmetric
+//     pair is searched once, by its lower endpoint, and counts for both.
+//   v unmatched: every entry (v, y), y != v, must have mate[y] set (an entry of
+//     a matched row is covered).
+// Counting rules are those of the host checker.
 //
-// Existence pass (check_pairs32), over 32 consecutive vertices: a vertex v
-// naming a partner m in range must share an edge with it, stored in row v or
-// in row m (the CSR may hold an edge for one endpoint only).  The warp
-// searches the shorter of the two rows first and stops at the first hit; a
-// symmetric pair is searched once, by its lower endpoint, and counts for
-// both.  Counting rules are those of the host checker.
+// The visit is bound by latency -- mate[v], then mate[m] and m's row ends, then
+// ids, then their mates -- and most rows it reads are a few entries long, so a
+// lane reads its own row, 8 entries a step, which keeps 32 rows in flight a
+// warp; a row of more than kLaneQuads quads is read by the whole warp, 256
+// entries a step.  A row of an unmatched vertex longer than kLongRow entries
+// (hubs, in matchings that are not maximal) is left to a second kernel that
+// spreads it over the GPU.
 #pragma once
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -21,132 +26,59 @@
 #include "state.cuh"
 
 namespace skp {
+
+// counters of one verdict, in mm_verdict's order after the flags.  The two
+// "first offender" fields hold the complement of the index and grow
+// (atomicMax), so that a block of zeros is a fresh set of counters.
+enum CheckSlot : int { kCkMatched = 0, kCkPairs, kCkRange, kCkAsym, kCkNonedge, kCkUncovered, kCkPairsBad,
+                       kCkFirstBad, kCkFirstUncovered, kCkCount,
+                       // control words behind them: long rows queued, blocks done
+                       kCkLong = kCkCount, kCkDone, kCkWords };
+constexpr int64_t kLongRow = 16384;  // entries; see above
+constexpr int kCheckBlocks = 5;      // resident blocks of 256 threads an SM of the checker's kernels
+
 namespace {
 
-__device__ __forceinline__ int check_count_le(int rel, int p) {
-  int c = 0;
-#pragma unroll
-  for (int step = 16; step >= 1; step >>= 1) {
-    const int v = __shfl_sync(kFull, rel, c + step - 1);
-    if (v <= p) c += step;
+constexpr int64_t kLaneQuads = 8;
+
+// a graph as the checker reads it (nbrs 16-byte aligned, nnz entries in all)
+struct CheckView {
+  const int64_t* offsets;
+  const uint32_t* nbrs;
+  const uint32_t* mate;
+  uint64_t n, nnz;
+};
+
+// what one visit found: the vertex's bits, and the uncovered entries this lane met
+enum : uint32_t { kVxMatched = 1u, kVxPair = 2u, kVxRange = 4u, kVxAsym = 8u, kVxNonedge = 16u,
+                  kVxBothEnds = 32u /* a missing edge of a symmetric pair: counts for both ends */,
+                  kVxBad = kVxRange | kVxAsym | kVxNonedge };
+struct Visit {
+  uint32_t bits = 0, uncovered = 0;
+  unsigned long long first_unc = ~0ull;
+};
+
+// rows of unmatched vertices left to the second kernel: graph << 32 | vertex
+struct LongRows {
+  unsigned long long* count;
+  uint64_t* items;
+};
+
+// last g < G with base[g] <= x (base ascending, base[0] = 0 <= x < base[G]), found by the whole warp
+template <class T>
+__device__ __forceinline__ uint64_t warp_last_at_or_below(const T* base, uint64_t G, uint64_t x, unsigned lane) {
+  uint64_t lo = 0, hi = G;
+  while (hi - lo > 1) {
+    const uint64_t step = (hi - lo + 31) / 32, at = lo + lane * step;
+    const unsigned below = __ballot_sync(kFull, at < hi && (uint64_t)__ldg(base + at) <= x);
+    lo += (uint64_t)(__popc(below) - 1) * step;
+    hi = lo + step < hi ? lo + step : hi;
   }
-  return c;
+  return lo;
 }
 
-// Accumulates, per lane, the uncovered entries and the smallest such index.
-__device__ __forceinline__ void check_unit(const int64_t* __restrict__ offsets,
-                                           const uint32_t* __restrict__ nbrs, uint64_t n,
-                                           uint64_t nnz, const uint32_t* __restrict__ mate,
-                                           int64_t row0, int64_t pos, const int64_t e_end,
-                                           const unsigned lane, unsigned long long& unc,
-                                           unsigned long long& first_unc) {
-  int64_t wbase = row0;
-  int64_t my_end = 0;
-  uint32_t my_mate = kNone;
-  unsigned busy = 0;  // rows of the window whose mate is set: none of their entries is uncovered
-  bool need = true;
-  while (pos < e_end) {
-    if (need) {
-      const int64_t r = wbase + lane;
-      const bool in = r < (int64_t)n;
-      my_end = in ? __ldg(offsets + r + 1) : INT64_MAX;
-      my_mate = in ? __ldg(mate + r) : kNone;
-      busy = __ballot_sync(kFull, !in || my_mate != kNone);
-      need = false;
-    }
-    const unsigned open = __ballot_sync(kFull, my_end > pos) & ~busy;
-    const int64_t win_end = __shfl_sync(kFull, my_end, 31);
-    if (open == 0u) {  // nothing left to check in this window
-      if (win_end >= e_end) return;
-      if (win_end > pos) pos = win_end;
-      wbase += 32;
-      need = true;
-      continue;
-    }
-    const int k1 = __ffs(open) - 1;
-    if (k1 > 0) {  // row k1 starts where row k1-1 ends
-      const int64_t st = __shfl_sync(kFull, my_end, k1 - 1);
-      if (st > pos) pos = st;
-    }
-    if (pos >= e_end) return;
-    const int64_t base = pos & ~(int64_t)3;
-    int64_t cend = base + 128;
-    if (cend > e_end) cend = e_end;
-    if (cend > win_end) cend = win_end;
-    const int lo_r = (int)(pos - base), hi_r = (int)(cend - base);
-    const int64_t rel64 = my_end - base;
-    const int rel = rel64 < 0 ? -1 : (rel64 > 129 ? 129 : (int)rel64);
-    const int p0 = 4 * (int)lane;
-    const int64_t e0 = base + p0;
-    uint32_t y[4] = {0u, 0u, 0u, 0u};
-    if (p0 < hi_r) {
-      if (e0 + 4 <= (int64_t)nnz) {
-        const uint4 q = __ldg(reinterpret_cast<const uint4*>(nbrs + e0));
-        y[0] = q.x; y[1] = q.y; y[2] = q.z; y[3] = q.w;
-      } else {
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (e0 + j < (int64_t)nnz) y[j] = __ldg(nbrs + e0 + j);
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int k = check_count_le(rel, p0 + j);
-      const int p = p0 + j;
-      if (p < lo_r || p >= hi_r || (busy >> (k & 31) & 1u)) continue;
-      const uint32_t x = (uint32_t)(wbase + k);
-      if (y[j] == x || y[j] >= n) continue;
-      if (__ldg(mate + y[j]) == kNone) {
-        ++unc;
-        const unsigned long long e = (unsigned long long)(e0 + j);
-        if (e < first_unc) first_unc = e;
-      }
-    }
-    pos = cend;
-  }
-}
-
-// Does row r hold the id t?  The whole warp reads the row, 32 entries a step.
-__device__ __forceinline__ bool warp_row_has(const int64_t* __restrict__ offsets,
-                                             const uint32_t* __restrict__ nbrs, uint32_t r,
-                                             uint32_t t, unsigned lane) {
-  const int64_t s = __ldg(offsets + r), e = __ldg(offsets + r + 1);
-  for (int64_t i = s; i < e; i += 32) {
-    const int64_t k = i + lane;
-    if (__any_sync(kFull, k < e && __ldg(nbrs + k) == t)) return true;
-  }
-  return false;
-}
-
-// Existence pass for vertices [v0, v0 + 32) of one graph (lane i: vertex v0 + i).
-// Adds to `nonedge` (lane 0) the vertices whose named partner shares no edge
-// with them, and lowers `first_bad` to the smallest of them.
-__device__ __forceinline__ void check_pairs32(const int64_t* __restrict__ offsets,
-                                              const uint32_t* __restrict__ nbrs, uint64_t n,
-                                              const uint32_t* __restrict__ mate, uint64_t v0,
-                                              unsigned lane, unsigned long long& nonedge,
-                                              unsigned long long& first_bad) {
-  const uint64_t v = v0 + lane;
-  const uint32_t m = v < n ? __ldg(mate + v) : kNone;
-  const bool valid = m != kNone && m < n && m != v;
-  const bool sym = valid && __ldg(mate + m) == (uint32_t)v;
-  unsigned todo = __ballot_sync(kFull, valid && !(sym && m < v));
-  while (todo) {
-    const int j = __ffs(todo) - 1;
-    todo &= todo - 1;
-    const uint32_t vj = (uint32_t)__shfl_sync(kFull, (unsigned)v, j);
-    const uint32_t mj = __shfl_sync(kFull, m, j);
-    const bool sj = __shfl_sync(kFull, sym ? 1u : 0u, j) != 0u;
-    const int64_t dv = __ldg(offsets + vj + 1) - __ldg(offsets + vj);
-    const int64_t dm = __ldg(offsets + mj + 1) - __ldg(offsets + mj);
-    const bool v_first = dv <= dm;  // the shorter row first
-    bool hit = warp_row_has(offsets, nbrs, v_first ? vj : mj, v_first ? mj : vj, lane);
-    if (!hit) hit = warp_row_has(offsets, nbrs, v_first ? mj : vj, v_first ? vj : mj, lane);
-    if (!hit && lane == 0) {
-      nonedge += sj ? 2 : 1;
-      if (vj < first_bad) first_bad = vj;  // a symmetric pair is searched by its lower end
-    }
-  }
+__device__ __forceinline__ void lower(unsigned long long& first, unsigned long long at) {
+  if (at < first) first = at;
 }
 
 __device__ __forceinline__ unsigned long long warp_sum64(unsigned long long v) {
@@ -162,6 +94,234 @@ __device__ __forceinline__ unsigned long long warp_min64(unsigned long long v) {
     v = o < v ? o : v;
   }
   return v;
+}
+
+// the ids at [q, q + 4), q a multiple of 4, as far as they exist before `e` or lie in a whole quad
+__device__ __forceinline__ uint4 check_quad(const uint32_t* nbrs, uint64_t nnz, int64_t q, int64_t e) {
+  uint4 y = make_uint4(0u, 0u, 0u, 0u);
+  if (q >= e) return y;
+  if (q + 4 <= (int64_t)nnz) return __ldg(reinterpret_cast<const uint4*>(nbrs + q));
+  y.x = __ldg(nbrs + q);
+  if (q + 1 < e) y.y = __ldg(nbrs + q + 1);
+  if (q + 2 < e) y.z = __ldg(nbrs + q + 2);
+  return y;
+}
+
+__device__ __forceinline__ bool quad_has(const uint4& y, int64_t q, int64_t s, int64_t e, uint32_t t) {
+  return (y.x == t && q >= s && q < e) || (y.y == t && q + 1 >= s && q + 1 < e) ||
+         (y.z == t && q + 2 >= s && q + 2 < e) || (y.w == t && q + 3 >= s && q + 3 < e);
+}
+
+// entries of the quad in [s, e) that leave the edge {x, y} uncovered (x is unmatched)
+__device__ __forceinline__ void quad_scan(const uint4& y4, int64_t q, int64_t s, int64_t e, uint32_t x,
+                                          const uint32_t* mate, uint64_t n, Visit& a) {
+  const uint32_t y[4] = {y4.x, y4.y, y4.z, y4.w};
+  bool free_y[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const bool live = q + j >= s && q + j < e && y[j] != x && y[j] < n;
+    free_y[j] = live && __ldg(mate + (live ? y[j] : 0u)) == kNone;
+  }
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+    if (free_y[j]) {
+      ++a.uncovered;
+      lower(a.first_unc, (unsigned long long)(q + j));
+    }
+}
+
+// Does [s, e) hold the id t?  The whole warp reads, 256 entries a step.
+__device__ __forceinline__ bool warp_row_has(const uint32_t* nbrs, uint64_t nnz, int64_t s, int64_t e,
+                                             uint32_t t, unsigned lane) {
+  for (int64_t b = s & ~(int64_t)3; b < e; b += 256) {
+    const int64_t q = b + 4 * (int64_t)lane;
+    const uint4 y0 = check_quad(nbrs, nnz, q, e), y1 = check_quad(nbrs, nnz, q + 128, e);
+    if (__any_sync(kFull, quad_has(y0, q, s, e, t) || quad_has(y1, q + 128, s, e, t))) return true;
+  }
+  return false;
+}
+
+template <class T>
+__device__ __forceinline__ T* shfl_ptr(T* p, int j) {
+  return reinterpret_cast<T*>(__shfl_sync(kFull, reinterpret_cast<unsigned long long>(p), j));
+}
+
+// Vertex v of the graph V, one a lane (`in`: the lane has one); `graph` is the
+// graph's number in the queue.  kOne: all lanes read one graph, and an
+// uncovered entry may be counted by any lane.
+template <bool kOne>
+__device__ __forceinline__ Visit check_group(const CheckView& V, bool in, uint32_t v, uint32_t graph,
+                                             unsigned lane, const LongRows& queue) {
+  Visit a;
+  uint32_t m = kNone;
+  int64_t s = 0, e = 0;                    // what is left of the row to read
+  if (in) {
+    m = __ldg(V.mate + v);
+    s = __ldg(V.offsets + v);
+    e = __ldg(V.offsets + v + 1);
+  }
+  uint32_t t = m;                          // the id searched for in it
+  const uint32_t other = v ^ m;            // t ^ other: the row's own vertex
+  bool find = false, again = true;         // search for t; the other row is still to come
+  if (m != kNone) {
+    if (m >= V.n || m == v) {
+      a.bits = kVxRange;
+    } else {
+      const bool sym = __ldg(V.mate + m) == v;
+      a.bits = kVxMatched | (sym ? kVxBothEnds | (v < m ? kVxPair : 0u) : kVxAsym);
+      find = !sym || v < m;
+      if (find) {
+        const int64_t s2 = __ldg(V.offsets + m), e2 = __ldg(V.offsets + m + 1);
+        if (e2 - s2 < e - s) {             // the shorter row first
+          s = s2;
+          e = e2;
+          t = v;
+        }
+      }
+    }
+  }
+  bool todo = find || (in && m == kNone && s < e);
+  for (;;) {  // short rows: one a lane
+    const bool mine = todo && ((e + 3) >> 2) - (s >> 2) <= kLaneQuads;
+    if (!__any_sync(kFull, mine)) break;
+    if (!mine) continue;
+    const int64_t q = s & ~(int64_t)3;
+    const uint4 y0 = check_quad(V.nbrs, V.nnz, q, e), y1 = check_quad(V.nbrs, V.nnz, q + 4, e);
+    if (find) {
+      if (quad_has(y0, q, s, e, t) || quad_has(y1, q + 4, s, e, t)) {
+        todo = false;
+        continue;
+      }
+    } else {
+      quad_scan(y0, q, s, e, v, V.mate, V.n, a);
+      quad_scan(y1, q + 4, s, e, v, V.mate, V.n, a);
+    }
+    s = q + 8;
+    if (s < e) continue;
+    if (find && again) {
+      again = false;
+      s = __ldg(V.offsets + t);
+      e = __ldg(V.offsets + t + 1);
+      t ^= other;
+    } else {
+      todo = false;
+      if (find) a.bits |= kVxNonedge;
+    }
+  }
+  unsigned left = __ballot_sync(kFull, todo);
+  while (left) {  // longer rows: the warp reads one at a time
+    const int j = __ffs(left) - 1;
+    left &= left - 1;
+    const int64_t sj = __shfl_sync(kFull, s, j), ej = __shfl_sync(kFull, e, j);
+    const uint32_t* nbrs = kOne ? V.nbrs : shfl_ptr(V.nbrs, j);
+    const uint64_t nnz = kOne ? V.nnz : __shfl_sync(kFull, V.nnz, j);
+    if (__shfl_sync(kFull, find ? 1 : 0, j)) {
+      const uint32_t tj = __shfl_sync(kFull, t, j), oj = __shfl_sync(kFull, other, j);
+      bool hit = warp_row_has(nbrs, nnz, sj, ej, tj, lane);
+      if (!hit && __shfl_sync(kFull, again ? 1 : 0, j)) {
+        const int64_t* offsets = kOne ? V.offsets : shfl_ptr(V.offsets, j);
+        hit = warp_row_has(nbrs, nnz, __ldg(offsets + tj), __ldg(offsets + tj + 1), tj ^ oj, lane);
+      }
+      if (!hit && (int)lane == j) a.bits |= kVxNonedge;
+    } else if (ej - sj > kLongRow) {
+      if ((int)lane == j) queue.items[atomicAdd(queue.count, 1ull)] = (uint64_t)graph << 32 | v;
+    } else {
+      const uint32_t xj = __shfl_sync(kFull, v, j);
+      const uint32_t* mate = kOne ? V.mate : shfl_ptr(V.mate, j);
+      const uint64_t n = kOne ? V.n : __shfl_sync(kFull, V.n, j);
+      Visit row;
+      for (int64_t b = sj & ~(int64_t)3; b < ej; b += 256) {
+        const int64_t q = b + 4 * (int64_t)lane;
+        const uint4 y0 = check_quad(nbrs, nnz, q, ej), y1 = check_quad(nbrs, nnz, q + 128, ej);
+        quad_scan(y0, q, sj, ej, xj, mate, n, row);
+        quad_scan(y1, q + 128, sj, ej, xj, mate, n, row);
+      }
+      if (kOne) {
+        a.uncovered += row.uncovered;
+        lower(a.first_unc, row.first_unc);
+      } else if (__any_sync(kFull, row.uncovered != 0u)) {
+        const uint32_t total = __reduce_add_sync(kFull, row.uncovered);
+        const unsigned long long first = warp_min64(row.first_unc);
+        if ((int)lane == j) {
+          a.uncovered += total;
+          lower(a.first_unc, first);
+        }
+      }
+    }
+  }
+  return a;
+}
+
+__device__ __forceinline__ void add_nonzero(unsigned long long* c, unsigned long long v) {
+  if (v) atomicAdd(c, v);
+}
+
+// The faults of one visit, each lane's vertex reported as index `at`, into
+// counters that all lanes share (every lane takes part).
+__device__ __forceinline__ void add_faults(unsigned long long* c, const Visit& a, unsigned long long at,
+                                           unsigned lane) {
+  if (!__any_sync(kFull, (a.bits & kVxBad) != 0u || a.uncovered != 0u)) return;
+  const uint32_t range = __popc(__ballot_sync(kFull, a.bits & kVxRange));
+  const uint32_t asym = __popc(__ballot_sync(kFull, a.bits & kVxAsym));
+  const unsigned missing = __ballot_sync(kFull, a.bits & kVxNonedge);
+  const uint32_t nonedge = __popc(missing) + __popc(missing & __ballot_sync(kFull, a.bits & kVxBothEnds));
+  const uint32_t uncovered = __reduce_add_sync(kFull, a.uncovered);
+  const unsigned long long bad = warp_min64(a.bits & kVxBad ? at : ~0ull), unc = warp_min64(a.first_unc);
+  if (lane == 0) {
+    add_nonzero(c + kCkRange, range);
+    add_nonzero(c + kCkAsym, asym);
+    add_nonzero(c + kCkNonedge, nonedge);
+    add_nonzero(c + kCkUncovered, uncovered);
+    if (~bad) atomicMax(c + kCkFirstBad, ~bad);
+    if (~unc) atomicMax(c + kCkFirstUncovered, ~unc);
+  }
+}
+
+// One queued row, spread over the whole grid.
+__device__ __forceinline__ void check_long_row(const CheckView& V, uint32_t x, unsigned long long* c,
+                                               unsigned lane) {
+  const int64_t s = __ldg(V.offsets + x), e = __ldg(V.offsets + x + 1);
+  const int64_t step = 4 * (int64_t)gridDim.x * blockDim.x;
+  Visit a;  // an entry in 4 * step: 32 bits hold a lane's share
+  for (int64_t q = (s & ~(int64_t)3) + 4 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x); q < e; q += step)
+    quad_scan(check_quad(V.nbrs, V.nnz, q, e), q, s, e, x, V.mate, V.n, a);
+  add_faults(c, a, 0, lane);
+}
+
+// A block's matched vertices and pairs (each warp's on all its lanes), added
+// once a block: added a warp at a time, the counts of 16.8 M vertices took
+// most of a 0.69 ms pass.
+__device__ __forceinline__ void add_block(unsigned long long* c, uint32_t matched, uint32_t pairs) {
+  __shared__ uint32_t sum[2][32];
+  const unsigned warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  if ((threadIdx.x & 31u) == 0) {
+    sum[0][warp] = matched;
+    sum[1][warp] = pairs;
+  }
+  __syncthreads();
+  if (threadIdx.x < 2) {
+    unsigned long long t = 0;
+    for (unsigned w = 0; w < nw; ++w) t += sum[threadIdx.x][w];
+    add_nonzero(c + (threadIdx.x ? kCkPairs : kCkMatched), t);
+  }
+}
+
+// The last block of the launch to get here writes the finished counters to
+// page-locked host memory and leaves the device's zeroed for the next check:
+// no launch before to clear them, no copy after to fetch them.
+__device__ __forceinline__ void publish_counters(unsigned long long* c, unsigned long long* host) {
+  __shared__ bool last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(c + kCkDone, 1ull) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  if (threadIdx.x < kCkWords) {
+    const unsigned long long v = atomicExch(c + threadIdx.x, 0ull);
+    if (threadIdx.x < kCkCount) host[threadIdx.x] = threadIdx.x >= kCkFirstBad ? ~v : v;
+  }
+  __threadfence_system();
 }
 
 }  // namespace

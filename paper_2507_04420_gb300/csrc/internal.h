@@ -46,16 +46,16 @@ struct BatchParams {
 };
 struct BatchKernels {
   const void* plan;        // <<<1, batch_plan_threads()>>>(BatchParams)
-  const void* prepare;     // (BatchParams, int states)
+  const void* prepare;     // (BatchParams)
   const void* sweep;       // (BatchParams); the serial kernel takes one warp per graph
   const void* pairs;       // (BatchParams)
 };
 void get_batch_kernels(int bits, bool local, bool serial, bool sym, bool lean, BatchKernels* k);
 int batch_sweep_blocks_per_sm(int bits, bool local, bool sym, bool lean, int block_threads);
 int batch_plan_threads();
-// one verdict for the whole batch in 9 counters (mm_verdict order after flags)
-cudaError_t launch_validate_batch(const BatchParams& B, unsigned long long* counters, int grid,
-                                  cudaStream_t s);
+// one verdict for the whole batch of graphs with local ids (cs as for launch_validate)
+struct CheckScratch;
+cudaError_t launch_validate_batch(const BatchParams& B, const CheckScratch& cs, int sms, cudaStream_t s);
 
 // coo.cu: Skipper over an edge list (src[i], dst[i]) in coordinate form
 struct CooParams {
@@ -77,25 +77,27 @@ void set_error_message(const char* fmt, ...);
 
 // check.cu
 struct CheckScratch {
-  unsigned long long* counters;  // mm_verdict-shaped device block (see check.cu)
+  unsigned long long* counters;  // kCkWords words, zero between checks (checkwalk.cuh)
+  unsigned long long* host;      // page-locked: the finished counters, in mm_verdict's order after the flags
   uint32_t* seen_bits;           // ceil(n/32) words
   uint64_t* block_counts;        // compaction: one count per tile of vertices
   uint64_t block_cap;
   unsigned char* found;          // edge-list checker: n bytes (+3), partner edge met in the list
-  int64_t* part;                 // checker: merge-path table, (n+nnz)/kCheckGrain + 1 pairs
+  uint64_t* long_rows;           // CSR checker: long_row_cap(nnz) entries, null when that is 0
 };
-constexpr uint64_t kCheckGrain = 4096;  // rows + entries per checker work unit
+uint64_t long_row_cap(uint64_t nnz);
+int check_grid(uint64_t n, int sms);
 cudaError_t launch_csr_check(uint64_t n, uint64_t nnz, const int64_t* offsets,
                              const uint32_t* nbrs, unsigned long long* bad, int grid,
                              cudaStream_t s);
 cudaError_t launch_validate(uint64_t n, uint64_t nnz, const int64_t* offsets, const uint32_t* nbrs,
                             const uint32_t* mate, const uint32_t* pairs, uint64_t count,
-                            const CheckScratch& cs, int grid, cudaStream_t s);
+                            const CheckScratch& cs, int sms, cudaStream_t s);
 cudaError_t launch_coo_check(uint64_t n, uint64_t m, const uint32_t* src, const uint32_t* dst,
                              unsigned long long* bad, int grid, cudaStream_t s);
 cudaError_t launch_validate_coo(uint64_t n, uint64_t m, const uint32_t* src, const uint32_t* dst,
                                 const uint32_t* mate, const uint32_t* pairs, uint64_t count,
-                                const CheckScratch& cs, int grid, cudaStream_t s);
+                                const CheckScratch& cs, int sms, cudaStream_t s);
 cudaError_t launch_census(const uint32_t* state, uint64_t n, int bits, unsigned long long* out,
                           int grid, cudaStream_t s);
 constexpr uint64_t kCompactTile = 4096;  // vertices per compaction tile

@@ -41,7 +41,7 @@ struct MultiParams {
   unsigned long long* work;
   uint32_t* err;
   uint64_t spin_limit;
-  unsigned long long* counters;  // checker: 9 per graph
+  unsigned long long* counters;  // checker: kCkCount per graph, then the long rows' count
 };
 
 // last g with base[g] <= x, base[0] = 0, base ascending, g < G
@@ -134,145 +134,76 @@ __global__ void multi_serial_kernel(MultiParams M) {
   serial_rows(S(P), P, 0, P.n, threadIdx.x & 31u);
 }
 
-enum { C_MATCHED = 0, C_PAIRS, C_RANGE, C_ASYM, C_NONEDGE, C_UNCOVERED, C_PAIRS_BAD, C_FIRST_BAD,
-       C_FIRST_UNCOVERED, C_N };
-
-__global__ void multi_counters_init_kernel(unsigned long long* c, uint64_t G) {
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < G * C_N;
-       i += (uint64_t)gridDim.x * blockDim.x)
-    c[i] = (i % C_N) >= C_FIRST_BAD ? ~0ull : 0ull;
-}
-
 __device__ __forceinline__ void group_add(unsigned long long* c, unsigned peers, uint32_t v) {
   const uint32_t s = __reduce_add_sync(peers, v);
   if ((int)(threadIdx.x & 31) == __ffs(peers) - 1 && s) atomicAdd(c, (unsigned long long)s);
 }
 
-__global__ void multi_partition_kernel(MultiParams M) {
-  const uint64_t G = M.num_graphs;
-  for (uint64_t u = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; u < M.units;
-       u += (uint64_t)gridDim.x * blockDim.x) {
-    const uint64_t g = find_graph(M.ubase, G, u);
-    const mm_graph_desc d = M.desc[g];
-    const int64_t total = (int64_t)(d.n + d.nnz);
-    int64_t diag = (int64_t)((u - M.ubase[g]) * M.grain);
-    if (diag > total) diag = total;
-    const int64_t rows = merge_path_rows(d.offsets, (int64_t)d.n, (int64_t)d.nnz, diag);
-    M.part[2 * u] = rows;
-    M.part[2 * u + 1] = diag - rows;
-    M.gid[u] = (uint32_t)g;
-  }
+// The exact checker (checkwalk.cuh) over every vertex of every graph, one set
+// of counters a graph.  A warp takes runs of kCheckRun * 32 consecutive
+// vertices of the whole batch: one search finds a run's graph, and its sums go
+// to the graph's counters when the run leaves it, not vertex by vertex.
+constexpr uint64_t kCheckRun = 8;
+
+__device__ __forceinline__ CheckView multi_check_view(const MultiParams& M, uint64_t g) {
+  const mm_graph_desc* d = M.desc + g;
+  return CheckView{d->offsets, d->nbrs, d->mate, d->n, d->nnz};
 }
 
-// the checker's edge pass (checkwalk.cuh) over the units of every graph
-__global__ void multi_validate_edges_kernel(MultiParams M) {
+__global__ void __launch_bounds__(256, kCheckBlocks) multi_check_kernel(MultiParams M, LongRows queue) {
   const unsigned lane = threadIdx.x & 31u;
   const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-  for (uint64_t u = warp; u < M.units; u += nwarps) {
-    const uint32_t g = M.gid[u];
-    const mm_graph_desc d = M.desc[g];
-    const int64_t e0 = M.part[2 * u + 1];
-    const int64_t e1 = (u + 1 < M.units && M.gid[u + 1] == g) ? M.part[2 * u + 3] : (int64_t)d.nnz;
-    if (e0 >= e1) continue;
-    unsigned long long unc = 0, first = ~0ull;
-    check_unit(d.offsets, d.nbrs, d.n, d.nnz, d.mate, M.part[2 * u], e0, e1, lane, unc, first);
-    unc = warp_sum64(unc);
-    first = warp_min64(first);
-    if (lane == 0) {
-      unsigned long long* c = M.counters + (uint64_t)g * C_N;
-      if (unc) atomicAdd(c + C_UNCOVERED, unc);
-      if (first != ~0ull) atomicMin(c + C_FIRST_UNCOVERED, first);
+  const uint64_t G = M.num_graphs, N = M.vbase[G];
+  for (uint64_t w0 = warp * 32 * kCheckRun; w0 < N; w0 += nwarps * 32 * kCheckRun) {
+    uint64_t g = warp_last_at_or_below(M.vbase, G, w0, lane);
+    uint64_t cur = g;  // the graph of the sums
+    uint32_t matched = 0, pairs = 0;
+    auto flush = [&]() {
+      if (lane == 0) {
+        add_nonzero(M.counters + cur * kCkCount + kCkMatched, matched);
+        add_nonzero(M.counters + cur * kCkCount + kCkPairs, pairs);
+      }
+      matched = pairs = 0;
+    };
+    for (uint64_t v0 = w0; v0 < w0 + 32 * kCheckRun && v0 < N; v0 += 32) {
+      const uint64_t i = v0 + lane;
+      const bool in = i < N;
+      while (in && i >= __ldg(M.vbase + g + 1)) ++g;
+      const uint32_t v = (uint32_t)(i - __ldg(M.vbase + g));
+      const Visit a = check_group<false>(multi_check_view(M, g), in, v, (uint32_t)g, lane, queue);
+      const uint64_t g0 = __shfl_sync(kFull, g, 0);
+      const unsigned active = __ballot_sync(kFull, in);
+      if (__all_sync(kFull, !in || g == g0)) {
+        if (g0 != cur) flush();
+        cur = g0;
+        matched += __popc(__ballot_sync(kFull, a.bits & kVxMatched));
+        pairs += __popc(__ballot_sync(kFull, a.bits & kVxPair));
+        add_faults(M.counters + g0 * kCkCount, a, v, lane);
+      } else if (in) {  // the group spans graphs: each lane counts for its own
+        unsigned long long* c = M.counters + g * kCkCount;
+        const unsigned peers = __match_any_sync(active, g);
+        group_add(c + kCkMatched, peers, a.bits & kVxMatched ? 1u : 0u);
+        group_add(c + kCkPairs, peers, a.bits & kVxPair ? 1u : 0u);
+        if (a.bits & kVxRange) atomicAdd(c + kCkRange, 1ull);
+        if (a.bits & kVxAsym) atomicAdd(c + kCkAsym, 1ull);
+        if (a.bits & kVxNonedge) atomicAdd(c + kCkNonedge, a.bits & kVxBothEnds ? 2ull : 1ull);
+        if (a.bits & kVxBad) atomicMax(c + kCkFirstBad, ~(unsigned long long)v);
+        add_nonzero(c + kCkUncovered, a.uncovered);
+        if (~a.first_unc) atomicMax(c + kCkFirstUncovered, ~a.first_unc);
+      }
+      g = __shfl_sync(kFull, g, 0);
     }
+    flush();
   }
 }
 
-// the checker's existence pass (checkwalk.cuh) over every vertex of every
-// graph: one warp per 32 consecutive vertices of the whole batch; the pairs
-// whose named edge is missing are counted in their graph's counters
-__global__ void multi_validate_exist_kernel(MultiParams M) {
-  const unsigned lane = threadIdx.x & 31u;
-  const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-  const uint64_t G = M.num_graphs;
-  const uint64_t V = M.vbase[G];
-  for (uint64_t w0 = warp * 32; w0 < V; w0 += nwarps * 32) {
-    const uint64_t gv = w0 + lane;
-    uint64_t g = 0;
-    uint32_t v = 0, m = kNone;
-    bool valid = false, sym = false;
-    if (gv < V) {
-      g = find_graph(M.vbase, G, gv);
-      const mm_graph_desc d = M.desc[g];
-      v = (uint32_t)(gv - M.vbase[g]);
-      m = d.mate[v];
-      valid = m != kNone && m < d.n && m != v;
-      sym = valid && d.mate[m] == v;
-    }
-    unsigned todo = __ballot_sync(kFull, valid && !(sym && m < v));
-    while (todo) {
-      const int j = __ffs(todo) - 1;
-      todo &= todo - 1;
-      const uint64_t gj = __shfl_sync(kFull, g, j);
-      const uint32_t vj = __shfl_sync(kFull, v, j), mj = __shfl_sync(kFull, m, j);
-      const bool sj = __shfl_sync(kFull, sym ? 1u : 0u, j) != 0u;
-      const mm_graph_desc d = M.desc[gj];
-      const int64_t dv = d.offsets[vj + 1] - d.offsets[vj];
-      const int64_t dm = d.offsets[mj + 1] - d.offsets[mj];
-      const bool v_first = dv <= dm;  // the shorter row first
-      bool hit = warp_row_has(d.offsets, d.nbrs, v_first ? vj : mj, v_first ? mj : vj, lane);
-      if (!hit) hit = warp_row_has(d.offsets, d.nbrs, v_first ? mj : vj, v_first ? vj : mj, lane);
-      if (!hit && lane == 0) {
-        unsigned long long* c = M.counters + gj * C_N;
-        atomicAdd(c + C_NONEDGE, sj ? 2ull : 1ull);
-        atomicMin(c + C_FIRST_BAD, (unsigned long long)vj);
-      }
-    }
-  }
-}
-
-// the checker's vertex pass on every vertex of every graph (range, symmetry,
-// pairs), counters kept per graph
-__global__ void multi_validate_kernel(MultiParams M) {
-  const uint64_t G = M.num_graphs;
-  const uint64_t V = M.vbase[G];
-  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  for (uint64_t v0 = (uint64_t)blockIdx.x * blockDim.x; v0 < V; v0 += stride) {
-    const uint64_t gv = v0 + threadIdx.x;
-    uint64_t g = ~0ull;
-    uint32_t matched = 0, pair = 0, range = 0, asym = 0;
-    uint64_t first_bad = ~0ull;
-    if (gv < V) {
-      g = find_graph(M.vbase, G, gv);
-      const mm_graph_desc d = M.desc[g];
-      const uint64_t v = gv - M.vbase[g];
-      const uint64_t n = d.n;
-      const uint32_t m = d.mate[v];
-      if (m != kNone) {
-        if (m >= n || m == v) {
-          range = 1;
-          first_bad = v;
-        } else {
-          matched = 1;
-          if (d.mate[m] != (uint32_t)v) {
-            asym = 1;
-            first_bad = v;
-          } else if (v < m) {
-            pair = 1;
-          }
-        }
-      }
-    }
-    const unsigned active = __ballot_sync(kFull, gv < V);
-    if (gv < V) {
-      const unsigned peers = __match_any_sync(active, g);
-      unsigned long long* c = M.counters + g * C_N;
-      group_add(c + C_MATCHED, peers, matched);
-      group_add(c + C_PAIRS, peers, pair);
-      group_add(c + C_RANGE, peers, range);
-      group_add(c + C_ASYM, peers, asym);
-      if (first_bad != ~0ull) atomicMin(c + C_FIRST_BAD, (unsigned long long)first_bad);
-    }
+__global__ void multi_check_long_kernel(MultiParams M, LongRows queue) {
+  const unsigned long long rows = *queue.count;
+  for (unsigned long long i = 0; i < rows; ++i) {
+    const uint64_t item = queue.items[i];
+    check_long_row(multi_check_view(M, item >> 32), (uint32_t)item, M.counters + (item >> 32) * kCkCount,
+                   threadIdx.x & 31u);
   }
 }
 
@@ -357,6 +288,7 @@ struct Layout {
   uint64_t bytes = 0;
   uint64_t off_ubase = 0, off_vbase = 0, off_sbase = 0;
   uint64_t total_vertices = 0, total_words = 0;
+  uint64_t long_rows = 0;              // rows that can be longer than kLongRow
 };
 
 mm_status stage_tables(TableSet* m, uint64_t G, const mm_graph_desc* h, uint64_t grain, int bits,
@@ -387,6 +319,7 @@ mm_status stage_tables(TableSet* m, uint64_t G, const mm_graph_desc* h, uint64_t
   for (uint64_t g = 0; g < G; ++g) {
     ub[g + 1] = ub[g] + (h[g].n + h[g].nnz + grain - 1) / grain;
     vb[g + 1] = vb[g] + h[g].n;
+    L->long_rows += long_row_cap(h[g].nnz);
     sb[g + 1] = sb[g] + (bits == 32 ? 0 : packed_words(h[g].n, bits) + 1);
   }
   L->units = ub[G];
@@ -539,34 +472,30 @@ mm_status mm_validate_multi_async(mm_multi* m, uint64_t num_graphs, const mm_gra
   if (st != MM_OK) return st;
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   Layout L;
-  if ((st = stage_tables(&m->check, num_graphs, h_descs, kCheckGrain, 32, s, &L)) != MM_OK) return st;
-  MTRY(grow(&m->counters, &m->counters_cap, num_graphs * C_N, s));
-  MTRY(grow(&m->check.part, &m->check.part_cap, 2 * (L.units + 1), s));
-  MTRY(grow(&m->check.gid, &m->check.gid_cap, L.units + 1, s));
-  if (m->h_counters_cap < num_graphs * C_N) {
+  if ((st = stage_tables(&m->check, num_graphs, h_descs, (uint64_t)kLongRow, 32, s, &L)) != MM_OK) return st;
+  const uint64_t words = num_graphs * kCkCount;
+  MTRY(grow(&m->counters, &m->counters_cap, words + 1, s));
+  MTRY(grow(&m->check.part, &m->check.part_cap, L.long_rows + 1, s));
+  if (m->h_counters_cap < words) {
     // the previous check's counters may still be on their way into the old buffer
     MTRY(cudaStreamSynchronize(s));
     if (m->h_counters) cudaFreeHost(m->h_counters);
     m->h_counters = nullptr;
-    uint64_t cap = m->h_counters_cap ? m->h_counters_cap : 64 * C_N;
-    while (cap < num_graphs * C_N) cap *= 2;
+    uint64_t cap = m->h_counters_cap ? m->h_counters_cap : 64 * kCkCount;
+    while (cap < words) cap *= 2;
     m->h_counters_cap = 0;
     MTRY(cudaMallocHost(&m->h_counters, cap * sizeof(unsigned long long)));
     m->h_counters_cap = cap;
   }
-  const MultiParams M = params(m, m->check, num_graphs, L, kCheckGrain, 1);
-  const int grid = m->num_sms * 8;
-  multi_counters_init_kernel<<<m->num_sms * 4, 256, 0, s>>>(m->counters, num_graphs);
+  const MultiParams M = params(m, m->check, num_graphs, L, (uint64_t)kLongRow, 1);
+  const LongRows queue{m->counters + words, reinterpret_cast<uint64_t*>(m->check.part)};
+  MTRY(cudaMemsetAsync(m->counters, 0, (words + 1) * sizeof(unsigned long long), s));
   if (L.total_vertices) {
-    if (L.units) {
-      multi_partition_kernel<<<grid, 256, 0, s>>>(M);
-      multi_validate_edges_kernel<<<grid, 256, 0, s>>>(M);
-    }
-    multi_validate_exist_kernel<<<grid, 256, 0, s>>>(M);
-    multi_validate_kernel<<<grid, 256, 0, s>>>(M);
+    multi_check_kernel<<<check_grid(L.total_vertices, m->num_sms), 256, 0, s>>>(M, queue);
+    if (L.long_rows) multi_check_long_kernel<<<m->num_sms * 2, 256, 0, s>>>(M, queue);
   }
   MTRY(cudaGetLastError());
-  MTRY(cudaMemcpyAsync(m->h_counters, m->counters, num_graphs * C_N * sizeof(unsigned long long),
+  MTRY(cudaMemcpyAsync(m->h_counters, m->counters, words * sizeof(unsigned long long),
                        cudaMemcpyDeviceToHost, s));
   m->checked_graphs = num_graphs;
   return MM_OK;
@@ -578,17 +507,17 @@ mm_status mm_multi_verdicts(mm_multi* m, uint64_t num_graphs, mm_verdict* h_out)
     return mfail(MM_ERR_ARG, "%llu verdicts asked, the last check covered %llu graphs",
                  (unsigned long long)num_graphs, (unsigned long long)m->checked_graphs);
   for (uint64_t g = 0; g < num_graphs; ++g) {
-    const unsigned long long* c = m->h_counters + g * C_N;
+    const unsigned long long* c = m->h_counters + g * kCkCount;
     mm_verdict v{};
-    v.n_matched = c[C_MATCHED];
-    v.n_pairs = c[C_PAIRS];
-    v.n_bad_range = c[C_RANGE];
-    v.n_asym = c[C_ASYM];
-    v.n_nonedge = c[C_NONEDGE];
-    v.n_uncovered = c[C_UNCOVERED];
+    v.n_matched = c[kCkMatched];
+    v.n_pairs = c[kCkPairs];
+    v.n_bad_range = c[kCkRange];
+    v.n_asym = c[kCkAsym];
+    v.n_nonedge = c[kCkNonedge];
+    v.n_uncovered = c[kCkUncovered];
     v.n_pairs_bad = 0;
-    v.first_bad_vertex = c[C_FIRST_BAD];
-    v.first_uncovered = c[C_FIRST_UNCOVERED];
+    v.first_bad_vertex = ~c[kCkFirstBad];
+    v.first_uncovered = ~c[kCkFirstUncovered];
     if (v.n_bad_range) v.flags |= MM_V_RANGE;
     if (v.n_asym) v.flags |= MM_V_ASYM;
     if (v.n_nonedge) v.flags |= MM_V_NONEDGE;
