@@ -1196,12 +1196,18 @@ mm_status mm_validate(mm_graph* g, const uint32_t* d_mate, const uint32_t* d_pai
     if (!g->found) CUDA_TRY(cudaMalloc(&g->found, g->n + 16));
     CUDA_TRY(launch_validate_coo(g->n, g->nnz, g->src, g->dst, d_mate, d_pairs, d_pairs ? count : 0,
                                  check_scratch(g), g->num_sms, s));
+    CUDA_TRY(cudaStreamSynchronize(s));
   } else {
     if ((st = ensure_long_rows(g)) != MM_OK) return st;
-    CUDA_TRY(launch_validate(g->n, g->nnz, g->offsets, g->nbrs, d_mate, d_pairs, d_pairs ? count : 0,
-                             check_scratch(g), g->num_sms, s));
+    const CheckScratch cs = check_scratch(g);
+    CUDA_TRY(launch_validate(g->n, g->nnz, g->offsets, g->nbrs, d_mate, d_pairs, d_pairs ? count : 0, cs,
+                             g->num_sms, s));
+    CUDA_TRY(cudaStreamSynchronize(s));
+    if (validate_needs_long(cs)) {
+      CUDA_TRY(launch_validate_long(g->n, g->nnz, g->offsets, g->nbrs, d_mate, cs, g->num_sms, s));
+      CUDA_TRY(cudaStreamSynchronize(s));
+    }
   }
-  CUDA_TRY(cudaStreamSynchronize(s));
   const unsigned long long* c = g->h_counters;
   mm_verdict v{};
   v.n_matched = c[0];
@@ -1235,6 +1241,7 @@ mm_status mm_validate_batched(mm_graph* g, uint64_t num_graphs, const int64_t* d
   if (!d_mate && g->n) return fail(MM_ERR_ARG, "null mate");
   if ((st = ensure_long_rows(g)) != MM_OK) return st;
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
+  const CheckScratch cs = check_scratch(g);
   if (g->local_ids) {
     BatchParams B{};
     B.P.n = g->n;
@@ -1244,12 +1251,20 @@ mm_status mm_validate_batched(mm_graph* g, uint64_t num_graphs, const int64_t* d
     B.P.mate = const_cast<uint32_t*>(d_mate);
     B.vbase = d_vbase;
     B.num_graphs = num_graphs;
-    CUDA_TRY(launch_validate_batch(B, check_scratch(g), g->num_sms, s));
+    CUDA_TRY(launch_validate_batch(B, cs, g->num_sms, s));
+    CUDA_TRY(cudaStreamSynchronize(s));
+    if (validate_needs_long(cs)) {
+      CUDA_TRY(launch_validate_batch_long(B, cs, g->num_sms, s));
+      CUDA_TRY(cudaStreamSynchronize(s));
+    }
   } else {  // no entry leaves its graph: the batch is checked as one CSR
-    CUDA_TRY(launch_validate(g->n, g->nnz, g->offsets, g->nbrs, d_mate, nullptr, 0, check_scratch(g),
-                             g->num_sms, s));
+    CUDA_TRY(launch_validate(g->n, g->nnz, g->offsets, g->nbrs, d_mate, nullptr, 0, cs, g->num_sms, s));
+    CUDA_TRY(cudaStreamSynchronize(s));
+    if (validate_needs_long(cs)) {
+      CUDA_TRY(launch_validate_long(g->n, g->nnz, g->offsets, g->nbrs, d_mate, cs, g->num_sms, s));
+      CUDA_TRY(cudaStreamSynchronize(s));
+    }
   }
-  CUDA_TRY(cudaStreamSynchronize(s));
   const unsigned long long* c = g->h_counters;
   mm_verdict v{};
   v.n_matched = c[0];

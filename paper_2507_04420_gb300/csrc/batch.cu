@@ -262,7 +262,7 @@ __global__ void batch_pairs_kernel(BatchParams B) {
 // the batch's.  (With global ids a batch is one CSR: launch_validate.)  A warp
 // takes runs of kCheckRun * 32 vertices, so that one search of vbase serves a
 // run and a lane then only steps on to the next graph. ----
-constexpr uint64_t kCheckRun = 8;
+constexpr uint64_t kCheckRun = 4;
 
 __device__ __forceinline__ CheckView batch_check_view(const BatchParams& B, uint64_t g) {
   const int64_t vb = __ldg(B.vbase + g);
@@ -285,14 +285,15 @@ __global__ void __launch_bounds__(256, kCheckBlocks) batch_check_kernel(BatchPar
       while (in && (int64_t)i >= __ldg(B.vbase + g + 1)) ++g;
       const CheckView V = batch_check_view(B, g);
       const uint64_t vb = (uint64_t)(V.mate - B.P.mate);
-      const Visit a = check_group<false>(V, in, (uint32_t)(i - vb), (uint32_t)g, lane, queue);
+      const uint32_t v = (uint32_t)(i - vb);
+      const Visit a = check_group<false>(V, in, v, load_vertex(V, in, v), (uint32_t)g, lane, queue);
       matched += __popc(__ballot_sync(kFull, a.bits & kVxMatched));
       pairs += __popc(__ballot_sync(kFull, a.bits & kVxPair));
       add_faults(c, a, i, lane);
     }
   }
   add_block(c, matched, pairs);
-  if (host) publish_counters(c, host);
+  publish_counters<false>(c, host);
 }
 
 __global__ void batch_check_long_kernel(BatchParams B, LongRows queue, unsigned long long* __restrict__ c,
@@ -302,7 +303,7 @@ __global__ void batch_check_long_kernel(BatchParams B, LongRows queue, unsigned 
     const uint64_t item = queue.items[i];
     check_long_row(batch_check_view(B, item >> 32), (uint32_t)item, c, threadIdx.x & 31u);
   }
-  publish_counters(c, host);
+  publish_counters<true>(c, host);
 }
 
 }  // namespace
@@ -344,9 +345,13 @@ int batch_sweep_blocks_per_sm(int bits, bool local, bool sym, bool lean, int blo
 
 cudaError_t launch_validate_batch(const BatchParams& B, const CheckScratch& cs, int sms, cudaStream_t s) {
   const LongRows queue{cs.counters + kCkLong, cs.long_rows};
-  const bool has_long = B.P.nnz > (uint64_t)kLongRow;
-  batch_check_kernel<<<check_grid(B.P.n, sms), 256, 0, s>>>(B, queue, cs.counters, has_long ? nullptr : cs.host);
-  if (has_long) batch_check_long_kernel<<<sms * 2, 256, 0, s>>>(B, queue, cs.counters, cs.host);
+  batch_check_kernel<<<check_grid(B.P.n, sms), 256, 0, s>>>(B, queue, cs.counters, cs.host);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_validate_batch_long(const BatchParams& B, const CheckScratch& cs, int sms, cudaStream_t s) {
+  batch_check_long_kernel<<<sms * 4, 256, 0, s>>>(B, LongRows{cs.counters + kCkLong, cs.long_rows}, cs.counters,
+                                                  cs.host);
   return cudaGetLastError();
 }
 

@@ -35,11 +35,12 @@ enum CheckSlot : int { kCkMatched = 0, kCkPairs, kCkRange, kCkAsym, kCkNonedge, 
                        // control words behind them: long rows queued, blocks done
                        kCkLong = kCkCount, kCkDone, kCkWords };
 constexpr int64_t kLongRow = 16384;  // entries; see above
-constexpr int kCheckBlocks = 5;      // resident blocks of 256 threads an SM of the checker's kernels
+constexpr int kCheckBlocks = 5;      // resident blocks of 256 threads an SM (4 and 6 are 5 to 10% slower)
 
 namespace {
 
-constexpr int64_t kLaneQuads = 8;
+// 8 / 16 / 32 quads: the 4096-graph batch's check 339 / 324 / 320 us, R-MAT 22's 170 / 174 / 185
+constexpr int64_t kLaneQuads = 16;
 
 // a graph as the checker reads it (nbrs 16-byte aligned, nnz entries in all)
 struct CheckView {
@@ -146,20 +147,29 @@ __device__ __forceinline__ T* shfl_ptr(T* p, int j) {
   return reinterpret_cast<T*>(__shfl_sync(kFull, reinterpret_cast<unsigned long long>(p), j));
 }
 
-// Vertex v of the graph V, one a lane (`in`: the lane has one); `graph` is the
+// Vertex v of the graph V with what load_vertex read of it, one a lane (`in`: the lane has one); `graph` is the
 // graph's number in the queue.  kOne: all lanes read one graph, and an
 // uncovered entry may be counted by any lane.
-template <bool kOne>
-__device__ __forceinline__ Visit check_group(const CheckView& V, bool in, uint32_t v, uint32_t graph,
-                                             unsigned lane, const LongRows& queue) {
-  Visit a;
-  uint32_t m = kNone;
-  int64_t s = 0, e = 0;                    // what is left of the row to read
+struct VertexRow {
+  uint32_t m = kNone;    // mate[v]
+  int64_t s = 0, e = 0;  // row v
+};
+__device__ __forceinline__ VertexRow load_vertex(const CheckView& V, bool in, uint32_t v) {
+  VertexRow r;
   if (in) {
-    m = __ldg(V.mate + v);
-    s = __ldg(V.offsets + v);
-    e = __ldg(V.offsets + v + 1);
+    r.m = __ldg(V.mate + v);
+    r.s = __ldg(V.offsets + v);
+    r.e = __ldg(V.offsets + v + 1);
   }
+  return r;
+}
+
+template <bool kOne>
+__device__ __forceinline__ Visit check_group(const CheckView& V, bool in, uint32_t v, const VertexRow& row,
+                                             uint32_t graph, unsigned lane, const LongRows& queue) {
+  Visit a;
+  const uint32_t m = row.m;
+  int64_t s = row.s, e = row.e;            // what is left of the row to read
   uint32_t t = m;                          // the id searched for in it
   const uint32_t other = v ^ m;            // t ^ other: the row's own vertex
   bool find = false, again = true;         // search for t; the other row is still to come
@@ -229,19 +239,19 @@ __device__ __forceinline__ Visit check_group(const CheckView& V, bool in, uint32
       const uint32_t xj = __shfl_sync(kFull, v, j);
       const uint32_t* mate = kOne ? V.mate : shfl_ptr(V.mate, j);
       const uint64_t n = kOne ? V.n : __shfl_sync(kFull, V.n, j);
-      Visit row;
+      Visit part;
       for (int64_t b = sj & ~(int64_t)3; b < ej; b += 256) {
         const int64_t q = b + 4 * (int64_t)lane;
         const uint4 y0 = check_quad(nbrs, nnz, q, ej), y1 = check_quad(nbrs, nnz, q + 128, ej);
-        quad_scan(y0, q, sj, ej, xj, mate, n, row);
-        quad_scan(y1, q + 128, sj, ej, xj, mate, n, row);
+        quad_scan(y0, q, sj, ej, xj, mate, n, part);
+        quad_scan(y1, q + 128, sj, ej, xj, mate, n, part);
       }
       if (kOne) {
-        a.uncovered += row.uncovered;
-        lower(a.first_unc, row.first_unc);
-      } else if (__any_sync(kFull, row.uncovered != 0u)) {
-        const uint32_t total = __reduce_add_sync(kFull, row.uncovered);
-        const unsigned long long first = warp_min64(row.first_unc);
+        a.uncovered += part.uncovered;
+        lower(a.first_unc, part.first_unc);
+      } else if (__any_sync(kFull, part.uncovered != 0u)) {
+        const uint32_t total = __reduce_add_sync(kFull, part.uncovered);
+        const unsigned long long first = warp_min64(part.first_unc);
         if ((int)lane == j) {
           a.uncovered += total;
           lower(a.first_unc, first);
@@ -308,7 +318,10 @@ __device__ __forceinline__ void add_block(unsigned long long* c, uint32_t matche
 
 // The last block of the launch to get here writes the finished counters to
 // page-locked host memory and leaves the device's zeroed for the next check:
-// no launch before to clear them, no copy after to fetch them.
+// no launch before to clear them, no copy after to fetch them.  With long rows
+// still queued (host[kCkLong] != 0) the counters stay as they are, for the
+// kernel that reads those rows (kFinal).
+template <bool kFinal>
 __device__ __forceinline__ void publish_counters(unsigned long long* c, unsigned long long* host) {
   __shared__ bool last;
   __threadfence();
@@ -317,9 +330,16 @@ __device__ __forceinline__ void publish_counters(unsigned long long* c, unsigned
   __syncthreads();
   if (!last) return;
   __threadfence();
-  if (threadIdx.x < kCkWords) {
-    const unsigned long long v = atomicExch(c + threadIdx.x, 0ull);
-    if (threadIdx.x < kCkCount) host[threadIdx.x] = threadIdx.x >= kCkFirstBad ? ~v : v;
+  const unsigned long long rows = kFinal ? 0ull : atomicAdd(c + kCkLong, 0ull);
+  if (threadIdx.x == 0) host[kCkLong] = rows;
+  if (rows) {
+    if (threadIdx.x == 0) c[kCkDone] = 0ull;
+  } else {
+    __syncthreads();  // every thread has read kCkLong
+    if (threadIdx.x < kCkWords) {
+      const unsigned long long v = atomicExch(c + threadIdx.x, 0ull);
+      if (threadIdx.x < kCkCount) host[threadIdx.x] = threadIdx.x >= kCkFirstBad ? ~v : v;
+    }
   }
   __threadfence_system();
 }

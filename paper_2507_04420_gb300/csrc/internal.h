@@ -56,6 +56,7 @@ int batch_plan_threads();
 // one verdict for the whole batch of graphs with local ids (cs as for launch_validate)
 struct CheckScratch;
 cudaError_t launch_validate_batch(const BatchParams& B, const CheckScratch& cs, int sms, cudaStream_t s);
+cudaError_t launch_validate_batch_long(const BatchParams& B, const CheckScratch& cs, int sms, cudaStream_t s);
 
 // coo.cu: Skipper over an edge list (src[i], dst[i]) in coordinate form
 struct CooParams {
@@ -93,6 +94,12 @@ cudaError_t launch_csr_check(uint64_t n, uint64_t nnz, const int64_t* offsets,
 cudaError_t launch_validate(uint64_t n, uint64_t nnz, const int64_t* offsets, const uint32_t* nbrs,
                             const uint32_t* mate, const uint32_t* pairs, uint64_t count,
                             const CheckScratch& cs, int sms, cudaStream_t s);
+// After launch_validate or launch_validate_batch has finished: rows of unmatched
+// vertices too long for one warp are left (a matching that is not maximal, as
+// a rule); the _long launch reads them and completes the counters.
+bool validate_needs_long(const CheckScratch& cs);
+cudaError_t launch_validate_long(uint64_t n, uint64_t nnz, const int64_t* offsets, const uint32_t* nbrs,
+                                 const uint32_t* mate, const CheckScratch& cs, int sms, cudaStream_t s);
 cudaError_t launch_coo_check(uint64_t n, uint64_t m, const uint32_t* src, const uint32_t* dst,
                              unsigned long long* bad, int grid, cudaStream_t s);
 cudaError_t launch_validate_coo(uint64_t n, uint64_t m, const uint32_t* src, const uint32_t* dst,
