@@ -84,10 +84,13 @@ typedef struct mm_options {
                                 list) per work unit.  Must be a multiple of 128
                                 when set.  0 = chosen from the graph: about two
                                 units per resident sweep warp, the nearest power
-                                of two in [512, 8192] (up to 32768 for
-                                MM_HOST_MAPPED handles, whose units each start by
-                                waiting on the host link).  mm_skipper_multi and
-                                mm_skipper_static take 0 as 2048. */
+                                of two in [512, 8192], at most 4096 where units are
+                                dispersed (2048 below 16 rows + entries a row,
+                                1024 below 8), up to 32768 for MM_HOST_MAPPED
+                                handles, whose units each start by waiting on the
+                                host link.  Batched and multi-graph calls choose
+                                from all their graphs together, down to 128.
+                                mm_skipper_static takes 0 as 2048. */
     uint32_t block_threads;  /* sweep threads per block, multiple of 32, <= 512;
                                 0 = 512 */
     uint32_t blocks_per_sm;  /* sweep blocks per SM; 0 = the occupancy maximum of the

@@ -143,7 +143,38 @@ struct Resolved {
   uint64_t spin_limit, poison;
 };
 
-mm_status resolve(const mm_graph* g, const mm_options* o, Resolved* r) {
+// Grain 0: about two units per resident warp, the nearest power of two between
+// two bounds (sweep times below in us, byte states).  Least 512 for one graph.
+// Most: per-unit costs against warps that run dry at the end.  Ascending units
+// 8192 (R-MAT 27: 4640, 4096 takes 4690).  Dispersed ones 4096 (2^26 edges of
+// factor 16: R-MAT 214, uniform 520; 8192 takes 229, 570), less where rows are
+// short: 2048 (R-MAT of edge factor 6: 343, 4096 takes 351, 1024 takes 459),
+// 1024 below 8 items a row (a 4096 x 4096 grid 804, 4096 takes 930).
+// Over the host link every unit's first window waits on the link: up to 32768.
+uint32_t grain_between(uint64_t items, uint64_t warps, uint64_t least, uint64_t most) {
+  const uint64_t target = items / (2 * warps);
+  uint64_t grain = least;
+  while (grain < most && grain * 1414 < target * 1000) grain *= 2;
+  return (uint32_t)grain;
+}
+uint64_t most_grain(uint64_t rows, uint64_t items, bool disperse) {
+  const uint64_t row = rows ? items / rows : 1;
+  return !disperse ? 8192 : row < 8 ? 1024 : row < 16 ? 2048 : 4096;
+}
+}  // namespace
+
+// The same for many graphs, whose units all start at once: a small batch's time
+// is one unit's chain of windows, so short rows take units down to 128 (64
+// graphs of 100 to 10,000 edges: 58 at 256, 70 at 512; 4096 mixed graphs: 953
+// at 2048, 8192 takes 1223).
+uint32_t skp::choose_grain(uint64_t rows, uint64_t items, uint64_t warps, bool disperse) {
+  const uint64_t row = rows ? items / rows : 1;
+  return grain_between(items, warps, row < 8 ? 128 : row < 24 ? 256 : 512, most_grain(rows, items, disperse));
+}
+
+namespace {
+
+mm_status resolve(const mm_graph* g, const mm_options* o, Resolved* r, bool batch = false) {
   mm_options d;
   mm_default_options(&d);
   if (!o) o = &d;
@@ -177,18 +208,12 @@ mm_status resolve(const mm_graph* g, const mm_options* o, Resolved* r) {
   r->lean = sweep_lean(r->bits, r->block, r->blocks_per_sm, fits);
   if (o->unit_order > MM_ORDER_DISPERSED) return fail(MM_ERR_ARG, "unit_order must be 0, 1 or 2 (got %u)", o->unit_order);
   r->disperse = o->unit_order == MM_ORDER_DISPERSED || (o->unit_order == MM_ORDER_AUTO && fits);
-  // grain 0: about two units per resident warp, the nearest power of two in
-  // [512, 8192] -- small graphs need many units to occupy the GPU, large ones
-  // lose to per-unit set-up below 4096; over the host link, where every
-  // unit's first window waits on the link, up to 32768
   if (r->grain == 0) {
-    const uint64_t items = g->coo ? g->nnz : g->n + g->nnz;
     const uint64_t warps = (uint64_t)(g->num_sms > 0 ? g->num_sms : 1) * (r->lean ? 64u : 48u);
-    const uint64_t target = items / (2 * warps);
-    const uint32_t cap = g->host_mapped ? 32768u : 8192u;
-    uint32_t grain = 512;
-    while (grain < cap && (uint64_t)grain * 1414 < target * 1000) grain *= 2;
-    r->grain = grain;
+    const uint64_t items = g->coo ? g->nnz : g->n + g->nnz;
+    const uint64_t most = g->host_mapped ? 32768 : g->coo ? 8192 : most_grain(g->n, items, r->disperse);
+    r->grain = batch && !g->host_mapped ? choose_grain(g->n, items, warps, r->disperse)
+                                        : grain_between(items, warps, 512, most);
   }
   r->spin_limit = o->spin_limit ? o->spin_limit : kDefaultSpin;
   r->poison = o->poison_vertex;
@@ -728,6 +753,7 @@ mm_status mm_skipper_to_host(mm_graph* g, const mm_options* o, uint32_t* d_mate,
       CUDA_TRY(cudaMemcpyAsync(work_ptr(g), hU + i, sizeof(uint64_t), cudaMemcpyHostToDevice, s));
     SweepParams Pi = P;
     Pi.units = (i + 1) * units / K;
+    Pi.first = hU[i];
     CUDA_TRY(launch_sweep(Pi, r.bits, grid, r.block, s));
     const uint64_t rows = i + 1 == K ? g->n : (hR[i + 1] < g->n ? hR[i + 1] : g->n);
     if (rows > done_rows) {
@@ -1122,7 +1148,7 @@ mm_status mm_skipper_batched(mm_graph* g, uint64_t num_graphs, const int64_t* d_
   if (!d_vbase || !d_ebase) return fail(MM_ERR_ARG, "null vbase / ebase");
   if (!d_mate && g->n) return fail(MM_ERR_ARG, "null mate");
   Resolved r;
-  if ((st = resolve(g, o, &r)) != MM_OK) return st;
+  if ((st = resolve(g, o, &r, true)) != MM_OK) return st;
   if (r.timing && r.use_graph) return fail(MM_ERR_UNSUPPORTED, "timing with use_graph");
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   if (g->local_ids || r.wpg)

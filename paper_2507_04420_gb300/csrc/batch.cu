@@ -194,11 +194,10 @@ __global__ void __launch_bounds__(512, kLean ? 4 : 3) batch_sweep_kernel(BatchPa
   const unsigned lane = threadIdx.x & 31u;
   const uint64_t pol = policy_evict_first();
   const uint64_t units = B.totals[0];
+  if (lane == 0) *warp_started() = 0u;
   const UnitOrder order(units, B.P.disperse != 0, (uint64_t)gridDim.x * (blockDim.x >> 5));
   for (;;) {
-    unsigned long long c = 0;
-    if (lane == 0) c = atomicAdd(B.P.work, 1ull);
-    c = __shfl_sync(kFull, c, 0);
+    const uint32_t c = take_unit(B.P.work, 0, lane);
     if (c >= order.total) return;
     const uint64_t w = order.unit(c);
     if (w >= units) continue;

@@ -77,10 +77,9 @@ __global__ void __launch_bounds__(512, 3) coo_sweep_kernel(CooParams C) {
   const S s(P);
   const uint64_t pol = policy_evict_first();
   const uint32_t n32 = (uint32_t)P.n;
+  if (lane == 0) *warp_started() = 0u;
   for (;;) {
-    unsigned long long w = 0;
-    if (lane == 0) w = atomicAdd(P.work, 1ull);
-    w = __shfl_sync(kFull, w, 0);
+    const uint64_t w = take_unit(P.work, 0, lane);
     if (w >= C.units) return;
     const uint64_t e_lo = w * C.grain;
     const uint64_t e_hi = e_lo + C.grain < C.m ? e_lo + C.grain : C.m;

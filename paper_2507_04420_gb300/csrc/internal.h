@@ -58,6 +58,10 @@ struct CheckScratch;
 cudaError_t launch_validate_batch(const BatchParams& B, const CheckScratch& cs, int sms, cudaStream_t s);
 cudaError_t launch_validate_batch_long(const BatchParams& B, const CheckScratch& cs, int sms, cudaStream_t s);
 
+// api.cu: rows + entries per work unit when the caller names none, for `warps`
+// resident warps
+uint32_t choose_grain(uint64_t rows, uint64_t items, uint64_t warps, bool disperse);
+
 // coo.cu: Skipper over an edge list (src[i], dst[i]) in coordinate form
 struct CooParams {
   SweepParams P;        // n, state, mate, work, err, spin_limit, poison, stats (CSR fields unused)

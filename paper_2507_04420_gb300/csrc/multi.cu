@@ -41,6 +41,7 @@ struct MultiParams {
   unsigned long long* work;
   uint32_t* err;
   uint64_t spin_limit;
+  uint32_t disperse;          // units handed out in dispersed runs
   unsigned long long* counters;  // checker: kCkCount per graph, then the long rows' count
 };
 
@@ -103,22 +104,24 @@ __global__ void multi_prepare_kernel(MultiParams M) {
   }
 }
 
-template <class S, bool kWord, bool kSel = false>
-__global__ void __launch_bounds__(512, 3) multi_sweep_kernel(MultiParams M) {
+template <class S, bool kWord, bool kSel = false, bool kLean = false>
+__global__ void __launch_bounds__(512, kLean ? 4 : 3) multi_sweep_kernel(MultiParams M) {
   const unsigned lane = threadIdx.x & 31u;
   const uint64_t pol = policy_evict_first();
+  if (lane == 0) *warp_started() = 0u;
+  const UnitOrder order(M.units, M.disperse != 0, (uint64_t)gridDim.x * (blockDim.x >> 5));
   for (;;) {
-    unsigned long long w = 0;
-    if (lane == 0) w = atomicAdd(M.work, 1ull);
-    w = __shfl_sync(kFull, w, 0);
-    if (w >= M.units) return;
+    const uint32_t c = take_unit(M.work, 0, lane);
+    if (c >= order.total) return;
+    const uint64_t w = order.unit(c);
+    if (w >= M.units) continue;
     const uint32_t g = M.gid[w];
     const SweepParams P = view(M, g, kWord);
     const int64_t row0 = M.part[2 * w];
     const int64_t e_begin = M.part[2 * w + 1];
     const int64_t e_end = (w + 1 < M.units && M.gid[w + 1] == g) ? M.part[2 * w + 3] : (int64_t)P.nnz;
     if (e_begin < e_end) sweep_unit<S, false, false, kSel>(S(P), P, row0, e_begin, e_end, lane, pol);
-    if ((w & 15) == 0) {
+    if ((c & 15) == 0) {
       uint32_t e = 0;
       if (lane == 0) e = ld_relaxed(M.err);
       if (__shfl_sync(kFull, e, 0) & kErrTimeout) return;
@@ -269,6 +272,7 @@ struct TableSet {
 struct mm_multi {
   int device = 0;
   int num_sms = 0;
+  int l2_bytes = 0;
   TableSet sweep, check;
   uint32_t* pool = nullptr;
   uint64_t pool_cap = 0;
@@ -376,6 +380,7 @@ mm_status mm_multi_create(mm_multi** out) {
   if (!m) return mfail(MM_ERR_OOM, "host allocation failed");
   cudaError_t e = cudaGetDevice(&m->device);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&m->num_sms, cudaDevAttrMultiProcessorCount, m->device);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&m->l2_bytes, cudaDevAttrL2CacheSize, m->device);
   if (e == cudaSuccess) e = cudaMalloc(&m->ctrl, 16 * sizeof(unsigned long long));
   if (e == cudaSuccess) e = cudaMallocHost(&m->h_err, 64);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&m->sweep.staging_free, cudaEventDisableTiming);
@@ -402,8 +407,8 @@ mm_status mm_skipper_multi(mm_multi* m, uint64_t num_graphs, const mm_graph_desc
   const uint32_t bits = o->status_bits ? o->status_bits : 8u;
   if (bits != 2 && bits != 8 && bits != 32) return mfail(MM_ERR_ARG, "status_bits must be 2, 8 or 32");
   const bool word = bits == 32;
-  const uint64_t grain = o->grain ? o->grain : 2048;
-  if (grain % 128 || grain > (1u << 24)) return mfail(MM_ERR_ARG, "bad grain");
+  if (o->grain % 128 || o->grain > (1u << 24)) return mfail(MM_ERR_ARG, "bad grain");
+  if (o->unit_order > MM_ORDER_DISPERSED) return mfail(MM_ERR_ARG, "unit_order must be 0, 1 or 2");
   const int block = o->block_threads ? (int)o->block_threads : 512;
   if (block < 32 || block > 512 || block % 32) return mfail(MM_ERR_ARG, "bad block_threads");
   if (o->id_loads > MM_ID_LOADS_SELECTIVE) return mfail(MM_ERR_ARG, "id_loads must be 0, 1 or 2");
@@ -412,12 +417,23 @@ mm_status mm_skipper_multi(mm_multi* m, uint64_t num_graphs, const mm_graph_desc
     return mfail(MM_ERR_UNSUPPORTED, "timing, use_graph, poison_vertex and l2_persist are not "
                                      "available in multi-graph calls");
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
+  // work split as for one graph of all their rows and entries
+  uint64_t rows = 0, items = 0;
+  for (uint64_t g = 0; g < num_graphs; ++g) {
+    rows += h_descs[g].n;
+    items += h_descs[g].n + h_descs[g].nnz;
+  }
+  const uint64_t state_bytes = word ? 4 * rows : rows * bits / 8;
+  const bool fits = 2 * state_bytes <= (uint64_t)m->l2_bytes;
+  const bool disperse = o->unit_order == MM_ORDER_DISPERSED || (o->unit_order == MM_ORDER_AUTO && fits);
+  const uint64_t grain = o->grain ? o->grain : choose_grain(rows, items, (uint64_t)m->num_sms * (fits ? 64 : 48), disperse);
   Layout L;
   if ((st = stage_tables(&m->sweep, num_graphs, h_descs, grain, (int)bits, s, &L)) != MM_OK) return st;
   MTRY(grow(&m->sweep.part, &m->sweep.part_cap, 2 * (L.units + 1), s));
   MTRY(grow(&m->sweep.gid, &m->sweep.gid_cap, L.units + 1, s));
   if (!word) MTRY(grow(&m->pool, &m->pool_cap, L.total_words + 1, s));
-  const MultiParams M = params(m, m->sweep, num_graphs, L, grain, o->spin_limit ? o->spin_limit : (1ull << 20));
+  MultiParams M = params(m, m->sweep, num_graphs, L, grain, o->spin_limit ? o->spin_limit : (1ull << 20));
+  M.disperse = disperse ? 1u : 0u;
 
   const int prep_grid = m->num_sms * 8;
   if (word) multi_prepare_kernel<true><<<prep_grid, 256, 0, s>>>(M);
@@ -430,23 +446,21 @@ mm_status mm_skipper_multi(mm_multi* m, uint64_t num_graphs, const mm_graph_desc
     else if (bits == 2) multi_serial_kernel<TwoBitState, false><<<grid, threads, 0, s>>>(M);
     else multi_serial_kernel<ByteState, false><<<grid, threads, 0, s>>>(M);
   } else if (L.units) {
+    // 64 warps an SM (32 registers) where the states stay in L2, as in the
+    // single-graph sweep; selective loads wait on the host link all the same
+    const bool lean = !sel && (o->blocks_per_sm ? o->blocks_per_sm > 3 : fits);
+    void (*kernel)(MultiParams) = nullptr;
+#define SKP_MULTI(S, W)                                                                    \
+  (sel ? multi_sweep_kernel<S, W, true> : lean ? multi_sweep_kernel<S, W, false, true>     \
+                                               : multi_sweep_kernel<S, W>)
+    kernel = bits == 32 ? SKP_MULTI(WordState, true) : bits == 2 ? SKP_MULTI(TwoBitState, false) : SKP_MULTI(ByteState, false);
+#undef SKP_MULTI
     int per_sm = (int)o->blocks_per_sm;
     if (per_sm <= 0) {
-      cudaError_t e = bits == 32 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, multi_sweep_kernel<WordState, true>, block, 0)
-                    : bits == 2  ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, multi_sweep_kernel<TwoBitState, false>, block, 0)
-                                 : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, multi_sweep_kernel<ByteState, false>, block, 0);
+      const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, 0);
       if (e != cudaSuccess || per_sm < 1) per_sm = 1;
     }
-    const int grid = m->num_sms * per_sm;
-    if (sel) {
-      if (bits == 32) multi_sweep_kernel<WordState, true, true><<<grid, block, 0, s>>>(M);
-      else if (bits == 2) multi_sweep_kernel<TwoBitState, false, true><<<grid, block, 0, s>>>(M);
-      else multi_sweep_kernel<ByteState, false, true><<<grid, block, 0, s>>>(M);
-    } else {
-      if (bits == 32) multi_sweep_kernel<WordState, true><<<grid, block, 0, s>>>(M);
-      else if (bits == 2) multi_sweep_kernel<TwoBitState, false><<<grid, block, 0, s>>>(M);
-      else multi_sweep_kernel<ByteState, false><<<grid, block, 0, s>>>(M);
-    }
+    kernel<<<m->num_sms * per_sm, block, 0, s>>>(M);
   }
   MTRY(cudaGetLastError());
   MTRY(cudaMemcpyAsync(m->h_err, M.err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));

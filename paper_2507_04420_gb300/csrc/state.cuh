@@ -42,7 +42,8 @@ struct SweepParams {
   int64_t* part;        // merge-path unit starts: (row, entry) for units+1 diagonals
   uint64_t units;
   uint64_t grain;
-  unsigned long long* work;  // next unit to hand out
+  unsigned long long* work;  // counter of the units handed out (take_unit)
+  uint64_t first;       // first unit of this launch
   uint32_t* err;
   uint64_t spin_limit;
   uint64_t poison;      // vertex + 1 left RESERVED after init (fault injection), 0 = off
@@ -79,6 +80,28 @@ struct UnitOrder {
         total(disperse ? R * L : units_) {}
   __device__ __forceinline__ uint64_t unit(uint64_t c) const { return R == 1 ? c : (c % R) * L + c / R; }
 };
+
+// The warp's next number in that order: the place of the warp in the grid
+// first, then numbers after those from the counter, which starts at `first`
+// too.  At about 1 ns an addition the counter alone keeps the last of 9728
+// warps waiting 10 us for its first unit.  Whether a warp has started is a word
+// in shared memory, as a register more spills the walk.  32 bits number the
+// units (of 128 items or more) of any graph that fits a machine's memory.
+__device__ __forceinline__ volatile uint32_t* warp_started() {
+  __shared__ uint32_t started[16];
+  return started + (threadIdx.x >> 5);
+}
+__device__ __forceinline__ uint32_t take_unit(unsigned long long* counter, uint64_t first, unsigned lane) {
+  uint32_t c = 0;
+  if (lane == 0) {
+    const uint32_t warps = blockDim.x >> 5;
+    volatile uint32_t* const started = warp_started();
+    c = *started ? gridDim.x * warps + atomicAdd(reinterpret_cast<uint32_t*>(counter), 1u)
+                 : (uint32_t)first + blockIdx.x * warps + (threadIdx.x >> 5);
+    *started = 1u;
+  }
+  return __shfl_sync(kFull, c, 0);
+}
 
 // Sweep statistics, kept only by the kStats kernel instances.  A conflict is a
 // failed CAS at Algorithm 1 line 11 or 14 (Section VI-E, Table II); a field CAS

@@ -91,11 +91,16 @@ __global__ void __launch_bounds__(512, kLean ? 4 : 3) sweep_kernel(SweepParams P
   const uint64_t pol = policy_evict_first();
   uint32_t phase = 0;   // parity of the warp's tile barrier (kTile)
   if (kTile) init_window_tile(lane);
+  if (kLean && lane == 0) *warp_started() = 0u;
   const UnitOrder order(P.units, P.disperse != 0, (uint64_t)gridDim.x * (blockDim.x >> 5));
   for (;;) {
-    unsigned long long c = 0;
-    if (lane == 0) c = atomicAdd(P.work, 1ull);
-    c = __shfl_sync(kFull, c, 0);
+    uint32_t c = 0;
+    if constexpr (kLean) {
+      c = take_unit(P.work, P.first, lane);
+    } else {  // its units are many and large: all from the counter, a register less
+      if (lane == 0) c = atomicAdd(reinterpret_cast<uint32_t*>(P.work), 1u);
+      c = __shfl_sync(kFull, c, 0);
+    }
     if (c >= order.total) return;
     const uint64_t w = order.unit(c);
     if (w >= P.units) continue;
