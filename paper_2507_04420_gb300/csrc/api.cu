@@ -11,6 +11,7 @@
 #include <new>
 #include <cuda_runtime.h>
 
+#include "chip.cuh"
 #include "internal.h"
 #include "skipper.h"
 
@@ -140,6 +141,7 @@ struct Resolved {
   uint32_t wpg;
   bool lean;          // the 32-register instance of the plain / symmetric sweep
   bool disperse;      // units handed out in dispersed runs
+  bool plain;         // grain, block, occupancy and unit order are the library's choice
   uint64_t spin_limit, poison;
 };
 
@@ -184,6 +186,8 @@ mm_status resolve(const mm_graph* g, const mm_options* o, Resolved* r, bool batc
   r->bits = (int)bits;
   r->word = bits == 32;
   r->serial = o->serial != 0;
+  r->plain = o->grain == 0 && (o->block_threads == 0 || o->block_threads == kDefaultBlock) &&
+             o->blocks_per_sm == 0 && o->unit_order == MM_ORDER_AUTO;
   r->grain = o->grain;
   if (r->grain % 128 || r->grain > (1u << 24))
     return fail(MM_ERR_ARG, "grain must be a multiple of 128 and at most 2^24 (got %u)", r->grain);
@@ -281,6 +285,15 @@ SweepParams make_params(mm_graph* g, const Resolved& r, uint32_t* d_mate) {
   P.lean = r.lean && !r.serial && !r.stats && !P.sel && !P.tile;
   P.disperse = r.disperse ? 1u : 0u;
   return P;
+}
+
+// Does one block with the states on the chip walk this graph (chip.cu)?  Not
+// when the call asks for what only the sweep has (serial order, statistics, an
+// injected reservation, per-kernel times, selective loads, staged windows, an L2
+// window, or a work split, block or occupancy of its own).
+bool chip_single(const mm_graph* g, const Resolved& r, const SweepParams& P) {
+  return r.plain && !r.serial && !r.stats && !r.poison && !r.timing && !r.l2_persist && !P.sel && !P.tile &&
+         g->n + g->nnz <= kChipSingleItems;
 }
 
 mm_status read_err(mm_graph* g, cudaStream_t s) {
@@ -674,6 +687,12 @@ mm_status mm_skipper(mm_graph* g, const mm_options* o, uint32_t* d_mate, uint32_
   CheckScratch cs = check_scratch(g);
   g->last_bits = r.bits;
   g->last_state = P.state;
+  if (chip_single(g, r, P)) {
+    CUDA_TRY(launch_chip_single(P, r.bits, g->h_err, s));
+    if (d_pairs || d_count) CUDA_TRY(launch_compact(g->n, d_mate, d_pairs, d_pairs ? cap : 0, d_count, cs, s));
+    if (r.nosync) return MM_OK;
+    return read_err(g, s);
+  }
   cudaEvent_t* ev = nullptr;
   if (r.timing) {
     if ((st = ensure_hist(g)) != MM_OK) return st;

@@ -214,7 +214,9 @@ __device__ __forceinline__ uint64_t policy_evict_first() {
 }
 
 // Bounded wait with exponential back-off.  Returns false when the wait has
-// run past its limit or another thread has already reported an error.
+// run past its limit or another thread has already reported an error.  kNear:
+// the states are in shared memory, where the holder needs tens of nanoseconds.
+template <bool kNear>
 struct Waiter {
   uint64_t polls = 0;
   uint32_t ns = 32;
@@ -225,8 +227,12 @@ struct Waiter {
       return false;
     }
     if ((polls & 63) == 0 && ld_relaxed(P.err) != 0) return false;
-    __nanosleep(ns);
-    ns = ns < 1024 ? ns * 2 : 1024;
+    if (kNear) {
+      __nanosleep(20);
+    } else {
+      __nanosleep(ns);
+      ns = ns < 1024 ? ns * 2 : 1024;
+    }
     return true;
   }
 };
@@ -238,6 +244,7 @@ struct Waiter {
 // a failed attempt costs no extra load.
 template <int kBits>
 struct PackedState {
+  static constexpr bool kNear = false;
   static constexpr uint32_t kPerWord = 32u / kBits;
   static constexpr uint32_t kMask = (1u << kBits) - 1u;
   uint32_t* words;
@@ -326,6 +333,7 @@ __host__ __device__ __forceinline__ uint64_t packed_words(uint64_t n, int bits) 
 }
 
 struct WordState {
+  static constexpr bool kNear = false;
   static constexpr uint32_t kPerWord = 1;
   uint32_t* words;
   __device__ explicit WordState(const SweepParams& P) : words(P.state) {}
@@ -370,7 +378,7 @@ __device__ __forceinline__ bool resolve_edge(const S& s, uint32_t x, uint32_t y,
   const bool x_low = x < y;                  // lines 8-9: lower id reserved first
   const uint32_t u = x_low ? x : y, v = x_low ? y : x;
   uint32_t ru = x_low ? rx : ry, rv = x_low ? ry : rx;
-  Waiter wt;
+  Waiter<S::kNear> wt;
   uint32_t cnf = 0;                          // conflicts on this entry (kStats only)
   bool result = false;
   for (;;) {
@@ -395,7 +403,7 @@ __device__ __forceinline__ bool resolve_edge(const S& s, uint32_t x, uint32_t y,
     bool won = false, gave_up = false;
     for (;;) {                               // lines 13-16, holding u
       if (s.try_claim(v, u, rv, P)) {
-        if (kStats) {
+        if constexpr (kStats) {
           atomicAdd(P.stats + kStTrans + 1, 1ull);  // ACC -> MCHD (v)
           s.commit_checked(u, v, P.stats);          // lines 15-16, RSVD -> MCHD (u)
         } else {
@@ -417,7 +425,7 @@ __device__ __forceinline__ bool resolve_edge(const S& s, uint32_t x, uint32_t y,
       result = true;
       break;
     }
-    if (kStats)
+    if constexpr (kStats)
       s.release_checked(u, P.stats);         // lines 17-18, RSVD -> ACC
     else
       s.release(u);                          // lines 17-18
