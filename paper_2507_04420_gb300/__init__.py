@@ -137,7 +137,7 @@ class Graph:
         if pairs:
             cap = cap if cap is not None else max(self.n // 2, 1)
             d_pairs = torch.empty((cap, 2), dtype=torch.int32, device=dev)
-            d_count = torch.zeros(1, dtype=torch.int64, device=dev)
+            d_count = torch.empty(1, dtype=torch.int64, device=dev)  # the call writes it in every case
         _check(lib.mm_skipper(self._h, ctypes.byref(o), _ptr(mate), _ptr(d_pairs),
                               cap if pairs else 0, _ptr(d_count), _stream_ptr(stream)),
                "mm_skipper")

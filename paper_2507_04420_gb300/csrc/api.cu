@@ -87,8 +87,7 @@ struct mm_graph {
   const uint32_t* last_state = nullptr;
   unsigned char* found = nullptr;      // checker scratch, allocated on first mm_validate
   uint64_t* long_rows = nullptr;
-  uint64_t* tile_counts = nullptr;
-  uint64_t tile_cap = 0;
+  uint64_t* tiles = nullptr;           // compaction words (compact_words)
   uint32_t* h_err = nullptr;           // pinned
   unsigned long long* h_counters = nullptr;  // pinned, 16 words
   cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
@@ -127,7 +126,7 @@ unsigned long long* counters_ptr(mm_graph* g) { return g->ctrl + 8; }
 unsigned long long* census_ptr(mm_graph* g) { return g->ctrl + 20; }
 
 CheckScratch check_scratch(mm_graph* g) {
-  return CheckScratch{counters_ptr(g), g->h_counters, g->seen_bits, g->tile_counts, g->tile_cap, g->found, g->long_rows};
+  return CheckScratch{counters_ptr(g), g->h_counters, g->seen_bits, g->found, g->long_rows};
 }
 
 struct Resolved {
@@ -455,8 +454,7 @@ mm_status new_handle(uint64_t n, uint64_t items, cudaStream_t s, mm_graph** out)
   if ((st = step(cudaMalloc(&g->ctrl, 32 * sizeof(unsigned long long)), "control words")) != MM_OK) return st;
   if ((st = step(cudaMemsetAsync(g->ctrl, 0, 32 * sizeof(unsigned long long), s), "control words")) != MM_OK)
     return st;
-  g->tile_cap = (n + kCompactTile - 1) / kCompactTile + 1;
-  if ((st = step(cudaMalloc(&g->tile_counts, g->tile_cap * sizeof(uint64_t)), "tiles")) != MM_OK) return st;
+  if ((st = step(cudaMalloc(&g->tiles, compact_words(n) * sizeof(uint64_t)), "tiles")) != MM_OK) return st;
   if ((st = step(cudaMallocHost(&g->h_err, 64), "pinned status")) != MM_OK) return st;
   if ((st = step(cudaMallocHost(&g->h_counters, 16 * sizeof(unsigned long long)), "pinned counters")) != MM_OK)
     return st;
@@ -509,6 +507,10 @@ mm_status skipper_coo(mm_graph* g, const Resolved& r, uint32_t* d_mate, uint32_t
   C.P.err = err_ptr(g);
   C.P.spin_limit = r.spin_limit;
   C.P.poison = r.poison;
+  if (d_pairs || d_count) {
+    C.P.tiles = g->tiles;
+    C.P.tile_words = compact_words(g->n);
+  }
   C.src = g->src;
   C.dst = g->dst;
   C.m = g->nnz;
@@ -521,7 +523,6 @@ mm_status skipper_coo(mm_graph* g, const Resolved& r, uint32_t* d_mate, uint32_t
     C.P.stats = g->stats;
     g->stats_valid = true;
   }
-  CheckScratch cs = check_scratch(g);
   g->last_bits = r.bits;
   g->last_state = C.P.state;
   cudaEvent_t* ev = nullptr;
@@ -542,7 +543,7 @@ mm_status skipper_coo(mm_graph* g, const Resolved& r, uint32_t* d_mate, uint32_t
     CUDA_TRY(launch_coo_serial(C, r.bits, s));
   }
   if (ev) CUDA_TRY(cudaEventRecord(ev[2], s));
-  if (d_pairs || d_count) CUDA_TRY(launch_compact(g->n, d_mate, d_pairs, d_pairs ? cap : 0, d_count, cs, s));
+  if (d_pairs || d_count) CUDA_TRY(launch_compact(g->n, d_mate, d_pairs, d_pairs ? cap : 0, d_count, g->tiles, err_ptr(g), s));
   if (ev) CUDA_TRY(cudaEventRecord(ev[3], s));
   CUDA_TRY(cudaMemcpyAsync(g->h_err, err_ptr(g), sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
   if (r.nosync) return MM_OK;
@@ -677,6 +678,10 @@ mm_status mm_skipper(mm_graph* g, const mm_options* o, uint32_t* d_mate, uint32_
   const uint64_t units = (g->n + g->nnz + r.grain - 1) / r.grain;
   if ((st = ensure_part(g, units)) != MM_OK) return st;
   SweepParams P = make_params(g, r, d_mate);
+  if (d_pairs || d_count) {
+    P.tiles = g->tiles;
+    P.tile_words = compact_words(g->n);
+  }
   g->stats_valid = false;
   if (r.stats && !r.serial) {
     if (!g->stats) CUDA_TRY(cudaMalloc(&g->stats, kStCount * sizeof(unsigned long long)));
@@ -684,12 +689,11 @@ mm_status mm_skipper(mm_graph* g, const mm_options* o, uint32_t* d_mate, uint32_
     g->stats_valid = true;
   }
 
-  CheckScratch cs = check_scratch(g);
   g->last_bits = r.bits;
   g->last_state = P.state;
   if (chip_single(g, r, P)) {
     CUDA_TRY(launch_chip_single(P, r.bits, g->h_err, s));
-    if (d_pairs || d_count) CUDA_TRY(launch_compact(g->n, d_mate, d_pairs, d_pairs ? cap : 0, d_count, cs, s));
+    if (d_pairs || d_count) CUDA_TRY(launch_compact(g->n, d_mate, d_pairs, d_pairs ? cap : 0, d_count, g->tiles, err_ptr(g), s));
     if (r.nosync) return MM_OK;
     return read_err(g, s);
   }
@@ -711,8 +715,7 @@ mm_status mm_skipper(mm_graph* g, const mm_options* o, uint32_t* d_mate, uint32_
   }
   if (ev) CUDA_TRY(cudaEventRecord(ev[2], s));
   if (d_pairs || d_count) {
-    uint64_t* cnt = d_count;
-    CUDA_TRY(launch_compact(g->n, d_mate, d_pairs, d_pairs ? cap : 0, cnt, cs, s));
+    CUDA_TRY(launch_compact(g->n, d_mate, d_pairs, d_pairs ? cap : 0, d_count, g->tiles, err_ptr(g), s));
   }
   if (ev) CUDA_TRY(cudaEventRecord(ev[3], s));
   CUDA_TRY(cudaMemcpyAsync(g->h_err, err_ptr(g), sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
@@ -1477,7 +1480,7 @@ mm_status mm_destroy(mm_graph* g) {
   if (g->found) cudaFree(g->found);
   if (g->stats) cudaFree(g->stats);
   if (g->long_rows) cudaFree(g->long_rows);
-  if (g->tile_counts) cudaFree(g->tile_counts);
+  if (g->tiles) cudaFree(g->tiles);
   if (g->h_err) cudaFreeHost(g->h_err);
   if (g->h_counters) cudaFreeHost(g->h_counters);
   for (auto& e : g->piece_ev)

@@ -177,103 +177,136 @@ __global__ void validate_pairs_kernel(uint64_t n, const uint32_t* __restrict__ m
 }
 
 // ---- ordered compaction of (u, mate[u]), u < mate[u] ----
+// One pass: a block takes the next tile of 4096 vertices (a ticket keeps the
+// tiles in order), counts its pairs, learns how many come before them from the
+// tiles before it -- each publishes its own count at once and the running total
+// as soon as it knows it, in one 64-bit word -- and writes them.  Bound by
+// memory: the mates are read once, in 128-bit loads, and the pairs written once.
+// R-MAT 27 (134 M vertices): 573 us as a count, a scan and a scatter that read
+// the mates twice, a thread 16 in a row; COMPACT_NOW us.
 constexpr int kCompactThreads = 256;
-constexpr int kPerThread = (int)(kCompactTile / kCompactThreads);  // 16
+static_assert(kCompactTile == 16 * kCompactThreads, "a thread takes four quads of a tile");
+constexpr uint64_t kTileOwn = 1ull << 62, kTileTotal = 2ull << 62, kTileValue = kTileOwn - 1;
+constexpr uint32_t kTilePolls = 1u << 24;
 
-__device__ __forceinline__ bool takes(const uint32_t* mate, uint64_t n, uint64_t u) {
-  if (u >= n) return false;
-  const uint32_t m = mate[u];
-  return m != kNone && m < n && u < m;
+__device__ __forceinline__ uint64_t ld_tile(const uint64_t* p) {
+  uint64_t v;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_tile(uint64_t* p, uint64_t v) {
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
-__global__ void compact_count_kernel(uint64_t n, const uint32_t* __restrict__ mate,
-                                     uint64_t* __restrict__ tile_counts) {
-  const uint64_t base = (uint64_t)blockIdx.x * kCompactTile + (uint64_t)threadIdx.x * kPerThread;
-  uint32_t cnt = 0;
-#pragma unroll
-  for (int i = 0; i < kPerThread; ++i) cnt += takes(mate, n, base + i);
-  __shared__ uint32_t warp_sums[kCompactThreads / 32];
-  const uint32_t ws = __reduce_add_sync(kFull, cnt);
-  if ((threadIdx.x & 31) == 0) warp_sums[threadIdx.x >> 5] = ws;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    uint64_t t = 0;
-    for (int w = 0; w < kCompactThreads / 32; ++w) t += warp_sums[w];
-    tile_counts[blockIdx.x] = t;
-  }
-}
-
-// exclusive scan of the tile counts in place (one block); total -> *count
-__global__ void compact_scan_kernel(uint64_t tiles, uint64_t* __restrict__ tile_counts,
-                                    uint64_t* __restrict__ count) {
-  __shared__ uint64_t carry_s;
-  __shared__ uint64_t warp_tot[32];
-  if (threadIdx.x == 0) carry_s = 0;
-  __syncthreads();
-  const unsigned lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (uint64_t b = 0; b < tiles; b += blockDim.x) {
-    const uint64_t i = b + threadIdx.x;
-    const uint64_t v = i < tiles ? tile_counts[i] : 0;
-    uint64_t x = v;  // inclusive warp scan
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const uint64_t y = __shfl_up_sync(kFull, x, d);
-      if ((int)lane >= d) x += y;
-    }
-    if (lane == 31) warp_tot[wid] = x;
-    __syncthreads();
-    if (wid == 0) {
-      uint64_t t = lane < nw ? warp_tot[lane] : 0;
-#pragma unroll
-      for (int d = 1; d < 32; d <<= 1) {
-        const uint64_t y = __shfl_up_sync(kFull, t, d);
-        if ((int)lane >= d) t += y;
+// pairs before tile t: the totals and counts of the tiles before it, 32 at a
+// time (the whole warp); a wait that runs out sets `err` and answers with less
+__device__ __forceinline__ uint64_t pairs_before(const uint64_t* tiles, int64_t t, unsigned lane, uint32_t* err) {
+  uint64_t before = 0;
+  for (int64_t p = t - 1; p >= 0; p -= 32) {
+    const int64_t i = p - lane;
+    uint64_t v = i >= 0 ? ld_tile(tiles + i) : kTileTotal;
+    for (uint32_t polls = 0; __any_sync(kFull, v <= kTileValue); ++polls) {
+      if (polls > kTilePolls) {
+        if (lane == 0) atomicOr(err, kErrTimeout);
+        return before;
       }
-      if (lane < nw) warp_tot[lane] = t;  // inclusive over warps
+      if (v <= kTileValue) v = ld_tile(tiles + i);
     }
-    __syncthreads();
-    const uint64_t before = carry_s + (wid ? warp_tot[wid - 1] : 0) + x - v;
-    if (i < tiles) tile_counts[i] = before;
-    __syncthreads();
-    if (threadIdx.x == 0) carry_s += warp_tot[nw - 1];
-    __syncthreads();
+    const unsigned known = __ballot_sync(kFull, v >= kTileTotal);
+    const int last = known ? __ffs(known) - 1 : 31;   // the nearest tile that knows its total
+    uint64_t x = (int)lane <= last ? v & kTileValue : 0;
+#pragma unroll
+    for (int d = 16; d >= 1; d >>= 1) x += __shfl_xor_sync(kFull, x, d);
+    before += x;
+    if (known) break;
   }
-  if (threadIdx.x == 0 && count) *count = carry_s;
+  return before;
 }
 
-__global__ void compact_scatter_kernel(uint64_t n, const uint32_t* __restrict__ mate,
-                                       const uint64_t* __restrict__ tile_offsets,
-                                       uint32_t* __restrict__ pairs, uint64_t cap) {
-  const uint64_t base = (uint64_t)blockIdx.x * kCompactTile + (uint64_t)threadIdx.x * kPerThread;
-  uint32_t flags = 0, cnt = 0;
+// state: [ticket | a word per tile], zero before the launch
+__global__ void __launch_bounds__(kCompactThreads) compact_kernel(uint64_t n, const uint32_t* __restrict__ mate,
+                                                                  uint32_t* __restrict__ pairs, uint64_t cap,
+                                                                  uint64_t* __restrict__ count,
+                                                                  uint64_t* __restrict__ state, uint32_t* err) {
+  __shared__ uint32_t tile_s;
+  __shared__ uint32_t sub[32];         // pairs before each 128 vertices of the tile
+  __shared__ uint64_t before_s;
+  const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  if (threadIdx.x == 0) tile_s = atomicAdd(reinterpret_cast<uint32_t*>(state), 1u);
+  __syncthreads();
+  const uint64_t t = tile_s, base = t * kCompactTile + 4 * threadIdx.x;
+  const bool wide = (reinterpret_cast<uintptr_t>(mate) & 15u) == 0;
+  uint32_t m[4][4];
 #pragma unroll
-  for (int i = 0; i < kPerThread; ++i)
-    if (takes(mate, n, base + i)) {
-      flags |= 1u << i;
-      ++cnt;
+  for (int i = 0; i < 4; ++i) {        // quad i: vertices base + 1024 i on
+    const uint64_t u = base + 1024 * i;
+    if (wide && u + 4 <= n) {
+      const uint4 q = *reinterpret_cast<const uint4*>(mate + u);
+      m[i][0] = q.x; m[i][1] = q.y; m[i][2] = q.z; m[i][3] = q.w;
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) m[i][j] = u + j < n ? mate[u + j] : kNone;
     }
-  const unsigned lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  uint32_t x = cnt;
+  }
+  uint32_t take = 0, cnt = 0;          // a bit per vertex; a byte per quad
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (m[i][j] != kNone && m[i][j] < n && base + 1024 * i + j < m[i][j]) {
+        take |= 1u << (4 * i + j);
+        cnt += 1u << (8 * i);
+      }
+  uint32_t upto = cnt;                 // four sums over the lanes at once, each at most 128
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
-    const uint32_t y = __shfl_up_sync(kFull, x, d);
-    if ((int)lane >= d) x += y;
+    const uint32_t y = __shfl_up_sync(kFull, upto, d);
+    if ((int)lane >= d) upto += y;
   }
-  __shared__ uint32_t warp_tot[kCompactThreads / 32];
-  if (lane == 31) warp_tot[wid] = x;
-  __syncthreads();
-  uint32_t wbefore = 0;
-  for (unsigned w = 0; w < wid; ++w) wbefore += warp_tot[w];
-  uint64_t pos = tile_offsets[blockIdx.x] + wbefore + x - cnt;
+  if (lane == 31)
 #pragma unroll
-  for (int i = 0; i < kPerThread; ++i)
-    if (flags >> i & 1u) {
-      if (pos < cap) {
-        pairs[2 * pos] = (uint32_t)(base + i);
-        pairs[2 * pos + 1] = mate[base + i];
-      }
-      ++pos;
+    for (int i = 0; i < 4; ++i) sub[8 * i + warp] = upto >> (8 * i) & 255u;
+  __syncthreads();
+  if (warp == 0) {
+    const uint32_t own = sub[lane];
+    uint32_t x = own;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t y = __shfl_up_sync(kFull, x, d);
+      if ((int)lane >= d) x += y;
     }
+    sub[lane] = x - own;
+    const uint64_t total = __shfl_sync(kFull, x, 31);
+    uint64_t* tiles = state + 1;
+    if (lane == 0 && t) st_tile(tiles + t, kTileOwn | total);
+    const uint64_t before = pairs_before(tiles, (int64_t)t, lane, err);
+    if (lane == 0) {
+      st_tile(tiles + t, kTileTotal | (before + total));
+      before_s = before;
+      if (count && t == gridDim.x - 1) *count = before + total;
+    }
+  }
+  if (!pairs) return;
+  __syncthreads();
+  const bool wide_pairs = (reinterpret_cast<uintptr_t>(pairs) & 7u) == 0;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    uint64_t pos = before_s + sub[8 * i + warp] + ((upto - cnt) >> (8 * i) & 255u);
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (take >> (4 * i + j) & 1u) {
+        const uint32_t u = (uint32_t)(base + 1024 * i + j);
+        if (pos < cap) {
+          if (wide_pairs) {
+            *reinterpret_cast<uint2*>(pairs + 2 * pos) = make_uint2(u, m[i][j]);
+          } else {
+            pairs[2 * pos] = u;
+            pairs[2 * pos + 1] = m[i][j];
+          }
+        }
+        ++pos;
+      }
+  }
 }
 
 }  // namespace
@@ -375,18 +408,16 @@ cudaError_t launch_census(const uint32_t* state, uint64_t n, int bits, unsigned 
   return cudaGetLastError();
 }
 
-cudaError_t launch_compact(uint64_t n, const uint32_t* mate, uint32_t* pairs, uint64_t cap,
-                           uint64_t* count, const CheckScratch& cs, cudaStream_t s) {
-  const uint64_t tiles = (n + kCompactTile - 1) / kCompactTile;
-  if (tiles > cs.block_cap) return cudaErrorInvalidValue;
-  if (tiles == 0) {
+uint64_t compact_words(uint64_t n) { return (n + kCompactTile - 1) / kCompactTile + 1; }
+
+cudaError_t launch_compact(uint64_t n, const uint32_t* mate, uint32_t* pairs, uint64_t cap, uint64_t* count,
+                           uint64_t* state, uint32_t* err, cudaStream_t s) {
+  if (n == 0) {
     if (count) zero_u64_kernel<<<1, 32, 0, s>>>(reinterpret_cast<unsigned long long*>(count), 1, 0ull);
     return cudaGetLastError();
   }
-  compact_count_kernel<<<(unsigned)tiles, kCompactThreads, 0, s>>>(n, mate, cs.block_counts);
-  compact_scan_kernel<<<1, 1024, 0, s>>>(tiles, cs.block_counts, count);
-  if (pairs && cap)
-    compact_scatter_kernel<<<(unsigned)tiles, kCompactThreads, 0, s>>>(n, mate, cs.block_counts, pairs, cap);
+  compact_kernel<<<(unsigned)(compact_words(n) - 1), kCompactThreads, 0, s>>>(n, mate, cap ? pairs : nullptr, cap, count,
+                                                                             state, err);
   return cudaGetLastError();
 }
 

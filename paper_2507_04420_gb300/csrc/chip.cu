@@ -148,6 +148,7 @@ template <int kBits, bool kSym>
 __global__ void __launch_bounds__(kSingleThreads, 1) chip_single_kernel(SweepParams P, uint32_t* host_err) {
   __shared__ ChipShared sh;
   if (threadIdx.x == 0) *P.err = 0u;
+  for (uint64_t i = threadIdx.x; P.tiles && i < P.tile_words; i += blockDim.x) P.tiles[i] = 0ull;
   chip_graph<kBits, kSym>(P, sh, policy_evict_first());
   if (P.state != P.mate) {
     const uint32_t words = (uint32_t)packed_words(P.n, kBits);

@@ -44,6 +44,7 @@ __global__ void coo_prepare_kernel(CooParams C, int bits) {
       P.state[i] = (poison && i == pv / per) ? (kRsvd << ((pv % per) * (uint64_t)bits)) : 0u;
     for (uint64_t i = tid; i < n; i += nthreads) P.mate[i] = kNone;
   }
+  for (uint64_t i = tid; P.tiles && i < P.tile_words; i += nthreads) P.tiles[i] = 0ull;
   if (P.stats && tid < kStCount) P.stats[tid] = 0ull;
   if (tid == 0) {
     *P.work = 0ull;

@@ -85,8 +85,6 @@ struct CheckScratch {
   unsigned long long* counters;  // kCkWords words, zero between checks (checkwalk.cuh)
   unsigned long long* host;      // page-locked: the finished counters, in mm_verdict's order after the flags
   uint32_t* seen_bits;           // ceil(n/32) words
-  uint64_t* block_counts;        // compaction: one count per tile of vertices
-  uint64_t block_cap;
   unsigned char* found;          // edge-list checker: n bytes (+3), partner edge met in the list
   uint64_t* long_rows;           // CSR checker: long_row_cap(nnz) entries, null when that is 0
 };
@@ -112,7 +110,10 @@ cudaError_t launch_validate_coo(uint64_t n, uint64_t m, const uint32_t* src, con
 cudaError_t launch_census(const uint32_t* state, uint64_t n, int bits, unsigned long long* out,
                           int grid, cudaStream_t s);
 constexpr uint64_t kCompactTile = 4096;  // vertices per compaction tile
-cudaError_t launch_compact(uint64_t n, const uint32_t* mate, uint32_t* pairs, uint64_t cap,
-                           uint64_t* count, const CheckScratch& cs, cudaStream_t s);
+// state: compact_words(n) words, zero before the launch (the prepare kernels
+// zero them when SweepParams::tiles names them)
+uint64_t compact_words(uint64_t n);
+cudaError_t launch_compact(uint64_t n, const uint32_t* mate, uint32_t* pairs, uint64_t cap, uint64_t* count,
+                           uint64_t* state, uint32_t* err, cudaStream_t s);
 
 }  // namespace skp

@@ -47,6 +47,8 @@ struct SweepParams {
   uint32_t* err;
   uint64_t spin_limit;
   uint64_t poison;      // vertex + 1 left RESERVED after init (fault injection), 0 = off
+  uint64_t* tiles;      // compaction words to zero before the pass, or null
+  uint64_t tile_words;
   // batched serial mode
   const int64_t* vbase;
   uint64_t num_graphs;

@@ -72,6 +72,7 @@ __global__ void prepare_kernel(SweepParams P, uint64_t* graph_pairs, uint64_t nu
     P.part[2 * u + 1] = d - rows;
   }
   for (uint64_t g = tid; g < num_graphs && graph_pairs; g += nthreads) graph_pairs[g] = 0;
+  for (uint64_t i = tid; P.tiles && i < P.tile_words; i += nthreads) P.tiles[i] = 0ull;
   if (P.stats && tid < kStCount) P.stats[tid] = 0ull;
   if (tid == 0) {
     *P.work = 0ull;
