@@ -177,15 +177,17 @@ __global__ void validate_pairs_kernel(uint64_t n, const uint32_t* __restrict__ m
 }
 
 // ---- ordered compaction of (u, mate[u]), u < mate[u] ----
-// One pass: a block takes the next tile of 4096 vertices (a ticket keeps the
+// One pass: a block takes the next tile of 16384 vertices (a ticket keeps the
 // tiles in order), counts its pairs, learns how many come before them from the
 // tiles before it -- each publishes its own count at once and the running total
 // as soon as it knows it, in one 64-bit word -- and writes them.  Bound by
 // memory: the mates are read once, in 128-bit loads, and the pairs written once.
 // R-MAT 27 (134 M vertices): 573 us as a count, a scan and a scatter that read
-// the mates twice, a thread 16 in a row; COMPACT_NOW us.
-constexpr int kCompactThreads = 256;
-static_assert(kCompactTile == 16 * kCompactThreads, "a thread takes four quads of a tile");
+// the mates twice, a thread 16 in a row in all, 291 us so (4096-vertex
+// tiles: 381, the look back holds them up).
+constexpr int kCompactThreads = 512, kCompactQuads = 8, kCompactWarps = kCompactThreads / 32;
+static_assert(kCompactTile == 4 * kCompactQuads * kCompactThreads, "a thread takes eight quads of a tile");
+static_assert(kCompactQuads * kCompactWarps == 128, "a lane of the scan takes four of the tile's parts");
 constexpr uint64_t kTileOwn = 1ull << 62, kTileTotal = 2ull << 62, kTileValue = kTileOwn - 1;
 constexpr uint32_t kTilePolls = 1u << 24;
 
@@ -224,22 +226,22 @@ __device__ __forceinline__ uint64_t pairs_before(const uint64_t* tiles, int64_t 
 }
 
 // state: [ticket | a word per tile], zero before the launch
-__global__ void __launch_bounds__(kCompactThreads) compact_kernel(uint64_t n, const uint32_t* __restrict__ mate,
+__global__ void __launch_bounds__(kCompactThreads, 2) compact_kernel(uint64_t n, const uint32_t* __restrict__ mate,
                                                                   uint32_t* __restrict__ pairs, uint64_t cap,
                                                                   uint64_t* __restrict__ count,
                                                                   uint64_t* __restrict__ state, uint32_t* err) {
   __shared__ uint32_t tile_s;
-  __shared__ uint32_t sub[32];         // pairs before each 128 vertices of the tile
+  __shared__ __align__(16) uint32_t sub[128];   // pairs before each 128 vertices of the tile
   __shared__ uint64_t before_s;
   const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
   if (threadIdx.x == 0) tile_s = atomicAdd(reinterpret_cast<uint32_t*>(state), 1u);
   __syncthreads();
   const uint64_t t = tile_s, base = t * kCompactTile + 4 * threadIdx.x;
   const bool wide = (reinterpret_cast<uintptr_t>(mate) & 15u) == 0;
-  uint32_t m[4][4];
+  uint32_t m[kCompactQuads][4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {        // quad i: vertices base + 1024 i on
-    const uint64_t u = base + 1024 * i;
+  for (int i = 0; i < kCompactQuads; ++i) {  // quad i: vertices base + 2048 i on
+    const uint64_t u = base + 4 * kCompactThreads * i;
     if (wide && u + 4 <= n) {
       const uint4 q = *reinterpret_cast<const uint4*>(mate + u);
       m[i][0] = q.x; m[i][1] = q.y; m[i][2] = q.z; m[i][3] = q.w;
@@ -248,34 +250,40 @@ __global__ void __launch_bounds__(kCompactThreads) compact_kernel(uint64_t n, co
       for (int j = 0; j < 4; ++j) m[i][j] = u + j < n ? mate[u + j] : kNone;
     }
   }
-  uint32_t take = 0, cnt = 0;          // a bit per vertex; a byte per quad
+  uint32_t take = 0, cnt[2] = {0, 0};  // a bit per vertex; a byte per quad
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < kCompactQuads; ++i)
 #pragma unroll
     for (int j = 0; j < 4; ++j)
-      if (m[i][j] != kNone && m[i][j] < n && base + 1024 * i + j < m[i][j]) {
+      if (m[i][j] != kNone && m[i][j] < n && base + 4 * kCompactThreads * i + j < m[i][j]) {
         take |= 1u << (4 * i + j);
-        cnt += 1u << (8 * i);
+        cnt[i / 4] += 1u << (8 * (i % 4));
       }
-  uint32_t upto = cnt;                 // four sums over the lanes at once, each at most 128
+  uint32_t upto[2] = {cnt[0], cnt[1]};  // four sums over the lanes at once, each at most 128
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
-    const uint32_t y = __shfl_up_sync(kFull, upto, d);
-    if ((int)lane >= d) upto += y;
+    const uint32_t y0 = __shfl_up_sync(kFull, upto[0], d), y1 = __shfl_up_sync(kFull, upto[1], d);
+    if ((int)lane >= d) {
+      upto[0] += y0;
+      upto[1] += y1;
+    }
   }
   if (lane == 31)
 #pragma unroll
-    for (int i = 0; i < 4; ++i) sub[8 * i + warp] = upto >> (8 * i) & 255u;
+    for (int i = 0; i < kCompactQuads; ++i) sub[kCompactWarps * i + warp] = upto[i / 4] >> (8 * (i % 4)) & 255u;
   __syncthreads();
   if (warp == 0) {
-    const uint32_t own = sub[lane];
+    const uint4 part = reinterpret_cast<const uint4*>(sub)[lane];
+    const uint32_t own = part.x + part.y + part.z + part.w;
     uint32_t x = own;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
       const uint32_t y = __shfl_up_sync(kFull, x, d);
       if ((int)lane >= d) x += y;
     }
-    sub[lane] = x - own;
+    const uint32_t first = x - own;
+    reinterpret_cast<uint4*>(sub)[lane] =
+        make_uint4(first, first + part.x, first + part.x + part.y, first + part.x + part.y + part.z);
     const uint64_t total = __shfl_sync(kFull, x, 31);
     uint64_t* tiles = state + 1;
     if (lane == 0 && t) st_tile(tiles + t, kTileOwn | total);
@@ -290,12 +298,12 @@ __global__ void __launch_bounds__(kCompactThreads) compact_kernel(uint64_t n, co
   __syncthreads();
   const bool wide_pairs = (reinterpret_cast<uintptr_t>(pairs) & 7u) == 0;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    uint64_t pos = before_s + sub[8 * i + warp] + ((upto - cnt) >> (8 * i) & 255u);
+  for (int i = 0; i < kCompactQuads; ++i) {
+    uint64_t pos = before_s + sub[kCompactWarps * i + warp] + ((upto[i / 4] - cnt[i / 4]) >> (8 * (i % 4)) & 255u);
 #pragma unroll
     for (int j = 0; j < 4; ++j)
       if (take >> (4 * i + j) & 1u) {
-        const uint32_t u = (uint32_t)(base + 1024 * i + j);
+        const uint32_t u = (uint32_t)(base + 4 * kCompactThreads * i + j);
         if (pos < cap) {
           if (wide_pairs) {
             *reinterpret_cast<uint2*>(pairs + 2 * pos) = make_uint2(u, m[i][j]);

@@ -109,7 +109,7 @@ cudaError_t launch_validate_coo(uint64_t n, uint64_t m, const uint32_t* src, con
                                 const CheckScratch& cs, int sms, cudaStream_t s);
 cudaError_t launch_census(const uint32_t* state, uint64_t n, int bits, unsigned long long* out,
                           int grid, cudaStream_t s);
-constexpr uint64_t kCompactTile = 4096;  // vertices per compaction tile
+constexpr uint64_t kCompactTile = 16384;  // vertices per compaction tile
 // state: compact_words(n) words, zero before the launch (the prepare kernels
 // zero them when SweepParams::tiles names them)
 uint64_t compact_words(uint64_t n);

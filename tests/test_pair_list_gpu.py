@@ -1,5 +1,5 @@
 """The pair list (u, mate[u]), u < mate[u], in ascending u, at the edges of its
-tiles (4096 vertices, sub-blocks of 128), with more tiles than one look back
+tiles (16384 vertices, parts of 128), with more tiles than one look back
 covers, a mate array that is not 16-byte aligned, and room for fewer pairs."""
 import numpy as np
 import pytest
@@ -11,7 +11,7 @@ from tests.conftest import cuda_ok
 pytestmark = [pytest.mark.gpu, pytest.mark.skipif(not cuda_ok(), reason="needs a CUDA GPU")]
 
 
-@pytest.mark.parametrize("n", [1, 2, 127, 129, 1025, 4095, 4096, 4097, 8193, 40000, 700001])
+@pytest.mark.parametrize("n", [1, 2, 127, 129, 1025, 2047, 4097, 16383, 16384, 16385, 40000, 700001])
 def test_pairs_are_the_mates_in_order(n):
     import paper_2507_04420_gb300 as skp
     p = torch.from_numpy(np.random.RandomState(n).permutation(n))
