@@ -88,7 +88,7 @@ struct mm_graph {
   unsigned char* found = nullptr;      // checker scratch, allocated on first mm_validate
   uint64_t* long_rows = nullptr;
   uint64_t* tiles = nullptr;           // compaction words (compact_words)
-  uint32_t* h_err = nullptr;           // pinned
+  uint32_t* h_err = nullptr;           // pinned: [0] status of the last call, [1] of a call that waits
   unsigned long long* h_counters = nullptr;  // pinned, 16 words
   cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
   // event sets of timed calls, read back without blocking the calls themselves
@@ -295,9 +295,17 @@ bool chip_single(const mm_graph* g, const Resolved& r, const SweepParams& P) {
          g->n + g->nnz <= kChipSingleItems;
 }
 
-mm_status read_err(mm_graph* g, cudaStream_t s) {
+// The word a call that waits has its kernels report to; such calls on a handle
+// are one after the other.
+uint32_t* direct_err(mm_graph* g) {
+  g->h_err[1] = 0;
+  return g->h_err + 1;
+}
+
+mm_status read_err(mm_graph* g, cudaStream_t s, bool direct = false) {
   CUDA_TRY(cudaStreamSynchronize(s));
-  const uint32_t e = *g->h_err;
+  if (direct) g->h_err[0] = *static_cast<volatile uint32_t*>(g->h_err + 1);
+  const uint32_t e = *static_cast<volatile uint32_t*>(g->h_err);
   if (e & kErrTimeout) return fail(MM_ERR_TIMEOUT, "a wait on a reserved vertex ran past spin_limit");
   if (e & kErrBadId) return fail(MM_ERR_BAD_GRAPH, "a neighbour id >= n was met");
   return MM_OK;
@@ -511,6 +519,7 @@ mm_status skipper_coo(mm_graph* g, const Resolved& r, uint32_t* d_mate, uint32_t
     C.P.tiles = g->tiles;
     C.P.tile_words = compact_words(g->n);
   }
+  C.P.host_err = r.nosync ? nullptr : direct_err(g);
   C.src = g->src;
   C.dst = g->dst;
   C.m = g->nnz;
@@ -543,11 +552,11 @@ mm_status skipper_coo(mm_graph* g, const Resolved& r, uint32_t* d_mate, uint32_t
     CUDA_TRY(launch_coo_serial(C, r.bits, s));
   }
   if (ev) CUDA_TRY(cudaEventRecord(ev[2], s));
-  if (d_pairs || d_count) CUDA_TRY(launch_compact(g->n, d_mate, d_pairs, d_pairs ? cap : 0, d_count, g->tiles, err_ptr(g), s));
+  if (d_pairs || d_count) CUDA_TRY(launch_compact(g->n, d_mate, d_pairs, d_pairs ? cap : 0, d_count, g->tiles, err_ptr(g), C.P.host_err, s));
   if (ev) CUDA_TRY(cudaEventRecord(ev[3], s));
+  if (!r.nosync) return read_err(g, s, true);
   CUDA_TRY(cudaMemcpyAsync(g->h_err, err_ptr(g), sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-  if (r.nosync) return MM_OK;
-  return read_err(g, s);
+  return MM_OK;
 }
 
 }  // namespace
@@ -682,6 +691,7 @@ mm_status mm_skipper(mm_graph* g, const mm_options* o, uint32_t* d_mate, uint32_
     P.tiles = g->tiles;
     P.tile_words = compact_words(g->n);
   }
+  P.host_err = r.nosync ? nullptr : direct_err(g);
   g->stats_valid = false;
   if (r.stats && !r.serial) {
     if (!g->stats) CUDA_TRY(cudaMalloc(&g->stats, kStCount * sizeof(unsigned long long)));
@@ -692,10 +702,12 @@ mm_status mm_skipper(mm_graph* g, const mm_options* o, uint32_t* d_mate, uint32_
   g->last_bits = r.bits;
   g->last_state = P.state;
   if (chip_single(g, r, P)) {
-    CUDA_TRY(launch_chip_single(P, r.bits, g->h_err, s));
-    if (d_pairs || d_count) CUDA_TRY(launch_compact(g->n, d_mate, d_pairs, d_pairs ? cap : 0, d_count, g->tiles, err_ptr(g), s));
-    if (r.nosync) return MM_OK;
-    return read_err(g, s);
+    CUDA_TRY(launch_chip_single(P, r.bits, s));
+    if (d_pairs || d_count)
+      CUDA_TRY(launch_compact(g->n, d_mate, d_pairs, d_pairs ? cap : 0, d_count, g->tiles, err_ptr(g), P.host_err, s));
+    if (!r.nosync) return read_err(g, s, true);
+    CUDA_TRY(cudaMemcpyAsync(g->h_err, err_ptr(g), sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+    return MM_OK;
   }
   cudaEvent_t* ev = nullptr;
   if (r.timing) {
@@ -715,12 +727,12 @@ mm_status mm_skipper(mm_graph* g, const mm_options* o, uint32_t* d_mate, uint32_
   }
   if (ev) CUDA_TRY(cudaEventRecord(ev[2], s));
   if (d_pairs || d_count) {
-    CUDA_TRY(launch_compact(g->n, d_mate, d_pairs, d_pairs ? cap : 0, d_count, g->tiles, err_ptr(g), s));
+    CUDA_TRY(launch_compact(g->n, d_mate, d_pairs, d_pairs ? cap : 0, d_count, g->tiles, err_ptr(g), P.host_err, s));
   }
   if (ev) CUDA_TRY(cudaEventRecord(ev[3], s));
+  if (!r.nosync) return read_err(g, s, true);
   CUDA_TRY(cudaMemcpyAsync(g->h_err, err_ptr(g), sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-  if (r.nosync) return MM_OK;
-  return read_err(g, s);
+  return MM_OK;
 }
 
 mm_status mm_skipper_to_host(mm_graph* g, const mm_options* o, uint32_t* d_mate, uint32_t* h_mate,

@@ -182,9 +182,9 @@ __global__ void validate_pairs_kernel(uint64_t n, const uint32_t* __restrict__ m
 // tiles before it -- each publishes its own count at once and the running total
 // as soon as it knows it, in one 64-bit word -- and writes them.  Bound by
 // memory: the mates are read once, in 128-bit loads, and the pairs written once.
-// R-MAT 27 (134 M vertices): 573 us as a count, a scan and a scatter that read
-// the mates twice, a thread 16 in a row in all, 291 us so (4096-vertex
-// tiles: 381, the look back holds them up).
+// R-MAT 27 (134 M vertices): 573 us as a count, a scan and a scatter that read the
+// mates twice, a thread 16 in a row; 291 us in one pass (tiles of 4096 vertices:
+// 381, held up by the look back).
 constexpr int kCompactThreads = 512, kCompactQuads = 8, kCompactWarps = kCompactThreads / 32;
 static_assert(kCompactTile == 4 * kCompactQuads * kCompactThreads, "a thread takes eight quads of a tile");
 static_assert(kCompactQuads * kCompactWarps == 128, "a lane of the scan takes four of the tile's parts");
@@ -202,14 +202,15 @@ __device__ __forceinline__ void st_tile(uint64_t* p, uint64_t v) {
 
 // pairs before tile t: the totals and counts of the tiles before it, 32 at a
 // time (the whole warp); a wait that runs out sets `err` and answers with less
-__device__ __forceinline__ uint64_t pairs_before(const uint64_t* tiles, int64_t t, unsigned lane, uint32_t* err) {
+__device__ __forceinline__ uint64_t pairs_before(const uint64_t* tiles, int64_t t, unsigned lane, uint32_t* err,
+                                                 uint32_t* host_err) {
   uint64_t before = 0;
   for (int64_t p = t - 1; p >= 0; p -= 32) {
     const int64_t i = p - lane;
     uint64_t v = i >= 0 ? ld_tile(tiles + i) : kTileTotal;
     for (uint32_t polls = 0; __any_sync(kFull, v <= kTileValue); ++polls) {
       if (polls > kTilePolls) {
-        if (lane == 0) atomicOr(err, kErrTimeout);
+        if (lane == 0) report(err, host_err, kErrTimeout);
         return before;
       }
       if (v <= kTileValue) v = ld_tile(tiles + i);
@@ -229,7 +230,8 @@ __device__ __forceinline__ uint64_t pairs_before(const uint64_t* tiles, int64_t 
 __global__ void __launch_bounds__(kCompactThreads, 2) compact_kernel(uint64_t n, const uint32_t* __restrict__ mate,
                                                                   uint32_t* __restrict__ pairs, uint64_t cap,
                                                                   uint64_t* __restrict__ count,
-                                                                  uint64_t* __restrict__ state, uint32_t* err) {
+                                                                  uint64_t* __restrict__ state, uint32_t* err,
+                                                                     uint32_t* host_err) {
   __shared__ uint32_t tile_s;
   __shared__ __align__(16) uint32_t sub[128];   // pairs before each 128 vertices of the tile
   __shared__ uint64_t before_s;
@@ -287,7 +289,7 @@ __global__ void __launch_bounds__(kCompactThreads, 2) compact_kernel(uint64_t n,
     const uint64_t total = __shfl_sync(kFull, x, 31);
     uint64_t* tiles = state + 1;
     if (lane == 0 && t) st_tile(tiles + t, kTileOwn | total);
-    const uint64_t before = pairs_before(tiles, (int64_t)t, lane, err);
+    const uint64_t before = pairs_before(tiles, (int64_t)t, lane, err, host_err);
     if (lane == 0) {
       st_tile(tiles + t, kTileTotal | (before + total));
       before_s = before;
@@ -419,13 +421,13 @@ cudaError_t launch_census(const uint32_t* state, uint64_t n, int bits, unsigned 
 uint64_t compact_words(uint64_t n) { return (n + kCompactTile - 1) / kCompactTile + 1; }
 
 cudaError_t launch_compact(uint64_t n, const uint32_t* mate, uint32_t* pairs, uint64_t cap, uint64_t* count,
-                           uint64_t* state, uint32_t* err, cudaStream_t s) {
+                           uint64_t* state, uint32_t* err, uint32_t* host_err, cudaStream_t s) {
   if (n == 0) {
     if (count) zero_u64_kernel<<<1, 32, 0, s>>>(reinterpret_cast<unsigned long long*>(count), 1, 0ull);
     return cudaGetLastError();
   }
   compact_kernel<<<(unsigned)(compact_words(n) - 1), kCompactThreads, 0, s>>>(n, mate, cap ? pairs : nullptr, cap, count,
-                                                                             state, err);
+                                                                             state, err, host_err);
   return cudaGetLastError();
 }
 

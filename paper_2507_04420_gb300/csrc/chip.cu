@@ -67,7 +67,7 @@ struct ChipState {
       }
       cur = old;
       if (tries > P.spin_limit) {
-        atomicOr(P.err, kErrTimeout);
+        report(P.err, P.host_err, kErrTimeout);
         return false;
       }
     }
@@ -143,9 +143,9 @@ __device__ __forceinline__ void chip_graph(const SweepParams& P, ChipShared& sh,
 }
 
 // One graph, one launch.  P.state (packed layouts) receives the states as the
-// sweep would have left them; *host_err the pass's status.
+// sweep would have left them.
 template <int kBits, bool kSym>
-__global__ void __launch_bounds__(kSingleThreads, 1) chip_single_kernel(SweepParams P, uint32_t* host_err) {
+__global__ void __launch_bounds__(kSingleThreads, 1) chip_single_kernel(SweepParams P) {
   __shared__ ChipShared sh;
   if (threadIdx.x == 0) *P.err = 0u;
   for (uint64_t i = threadIdx.x; P.tiles && i < P.tile_words; i += blockDim.x) P.tiles[i] = 0ull;
@@ -154,23 +154,18 @@ __global__ void __launch_bounds__(kSingleThreads, 1) chip_single_kernel(SweepPar
     const uint32_t words = (uint32_t)packed_words(P.n, kBits);
     for (uint32_t i = threadIdx.x; i < words; i += blockDim.x) P.state[i] = g_chip_words[i];
   }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    *host_err = ld_relaxed(P.err);
-    __threadfence_system();
-  }
 }
 
 }  // namespace
 
-cudaError_t launch_chip_single(const SweepParams& P, int bits, uint32_t* host_err, cudaStream_t s) {
+cudaError_t launch_chip_single(const SweepParams& P, int bits, cudaStream_t s) {
   const int layout = bits == 2 ? 2 : 8;  // word states are the mates themselves: bytes on the chip
   const size_t bytes = 4 * (packed_words(P.n, layout) + 4);
   static_assert(kChipSingleItems + 16 <= (40u << 10), "the states of the largest graph fit without opting in to more");
-  void (*const kernel)(SweepParams, uint32_t*) =
+  void (*const kernel)(SweepParams) =
       layout == 2 ? (P.sym ? chip_single_kernel<2, true> : chip_single_kernel<2, false>)
                   : (P.sym ? chip_single_kernel<8, true> : chip_single_kernel<8, false>);
-  kernel<<<1, kSingleThreads, bytes, s>>>(P, host_err);
+  kernel<<<1, kSingleThreads, bytes, s>>>(P);
   return cudaGetLastError();
 }
 

@@ -10,7 +10,7 @@ namespace skp {
 // a grid of 39 K 93 / 91, 79 K 146 / 97.
 constexpr uint64_t kChipSingleItems = 32768;
 // the whole pass over one graph of at most that size: no prepare launch before
-// it, the status written to page-locked *host_err
-cudaError_t launch_chip_single(const SweepParams& P, int bits, uint32_t* host_err, cudaStream_t s);
+// it
+cudaError_t launch_chip_single(const SweepParams& P, int bits, cudaStream_t s);
 
 }  // namespace skp

@@ -114,6 +114,6 @@ constexpr uint64_t kCompactTile = 16384;  // vertices per compaction tile
 // zero them when SweepParams::tiles names them)
 uint64_t compact_words(uint64_t n);
 cudaError_t launch_compact(uint64_t n, const uint32_t* mate, uint32_t* pairs, uint64_t cap, uint64_t* count,
-                           uint64_t* state, uint32_t* err, cudaStream_t s);
+                           uint64_t* state, uint32_t* err, uint32_t* host_err, cudaStream_t s);
 
 }  // namespace skp

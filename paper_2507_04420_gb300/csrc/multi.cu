@@ -40,6 +40,7 @@ struct MultiParams {
   uint64_t grain;
   unsigned long long* work;
   uint32_t* err;
+  uint32_t* host_err;         // as SweepParams::host_err
   uint64_t spin_limit;
   uint32_t disperse;          // units handed out in dispersed runs
   unsigned long long* counters;  // checker: kCkCount per graph, then the long rows' count
@@ -65,6 +66,7 @@ __device__ __forceinline__ SweepParams view(const MultiParams& M, uint64_t g, bo
   P.mate = d.mate;
   P.state = word ? d.mate : M.state_pool + M.sbase[g];
   P.err = M.err;
+  P.host_err = M.host_err;
   P.spin_limit = M.spin_limit;
   return P;
 }
@@ -434,6 +436,8 @@ mm_status mm_skipper_multi(mm_multi* m, uint64_t num_graphs, const mm_graph_desc
   if (!word) MTRY(grow(&m->pool, &m->pool_cap, L.total_words + 1, s));
   MultiParams M = params(m, m->sweep, num_graphs, L, grain, o->spin_limit ? o->spin_limit : (1ull << 20));
   M.disperse = disperse ? 1u : 0u;
+  m->h_err[1] = 0;  // a call that waits has its kernels report here
+  M.host_err = o->nosync ? nullptr : m->h_err + 1;
 
   const int prep_grid = m->num_sms * 8;
   if (word) multi_prepare_kernel<true><<<prep_grid, 256, 0, s>>>(M);
@@ -463,15 +467,19 @@ mm_status mm_skipper_multi(mm_multi* m, uint64_t num_graphs, const mm_graph_desc
     kernel<<<m->num_sms * per_sm, block, 0, s>>>(M);
   }
   MTRY(cudaGetLastError());
-  MTRY(cudaMemcpyAsync(m->h_err, M.err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-  if (o->nosync) return MM_OK;
+  if (o->nosync) {
+    MTRY(cudaMemcpyAsync(m->h_err, M.err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+    return MM_OK;
+  }
+  MTRY(cudaStreamSynchronize(s));
+  m->h_err[0] = *static_cast<volatile uint32_t*>(m->h_err + 1);
   return mm_multi_sync(m, cuda_stream);
 }
 
 mm_status mm_multi_sync(mm_multi* m, void* cuda_stream) {
   if (!m) return mfail(MM_ERR_ARG, "null handle");
   MTRY(cudaStreamSynchronize(static_cast<cudaStream_t>(cuda_stream)));
-  const uint32_t e = *m->h_err;
+  const uint32_t e = *static_cast<volatile uint32_t*>(m->h_err);
   if (e & kErrTimeout) return mfail(MM_ERR_TIMEOUT, "a wait on a reserved vertex ran past spin_limit");
   if (e & kErrBadId) return mfail(MM_ERR_BAD_GRAPH, "a neighbour id >= n was met");
   return MM_OK;

@@ -45,6 +45,7 @@ struct SweepParams {
   unsigned long long* work;  // counter of the units handed out (take_unit)
   uint64_t first;       // first unit of this launch
   uint32_t* err;
+  uint32_t* host_err;   // the status word the host reads, or null (then `err` is copied to it)
   uint64_t spin_limit;
   uint64_t poison;      // vertex + 1 left RESERVED after init (fault injection), 0 = off
   uint64_t* tiles;      // compaction words to zero before the pass, or null
@@ -103,6 +104,14 @@ __device__ __forceinline__ uint32_t take_unit(unsigned long long* counter, uint6
     *started = 1u;
   }
   return __shfl_sync(kFull, c, 0);
+}
+
+// An error of the pass: into the device's word, which other warps look at, and,
+// where the host waits for the call, straight into page-locked memory, so that
+// no copy follows the pass.
+__device__ __forceinline__ void report(uint32_t* err, uint32_t* host_err, uint32_t bits) {
+  atomicOr(err, bits);
+  if (host_err) atomicOr_system(host_err, bits);
 }
 
 // Sweep statistics, kept only by the kStats kernel instances.  A conflict is a
@@ -225,7 +234,7 @@ struct Waiter {
   __device__ __forceinline__ bool wait(const SweepParams& P) {
     ++polls;
     if (polls > P.spin_limit) {
-      atomicOr(P.err, kErrTimeout);
+      report(P.err, P.host_err, kErrTimeout);
       return false;
     }
     if ((polls & 63) == 0 && ld_relaxed(P.err) != 0) return false;
@@ -288,7 +297,7 @@ struct PackedState {
       }
       cur = old;
       if (tries > P.spin_limit) {  // lock-free retry; bounded all the same
-        atomicOr(P.err, kErrTimeout);
+        report(P.err, P.host_err, kErrTimeout);
         return false;
       }
     }

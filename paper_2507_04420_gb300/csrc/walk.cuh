@@ -187,7 +187,7 @@ __device__ __forceinline__ void sweep_unit(const S& s, const SweepParams& P, int
       if (kTile && pending) {
         from_tile = wait_tile();
         if (!from_tile) {            // the copy did not land: stop, after a last bounded wait
-          if (lane == 0) atomicOr(P.err, kErrTimeout);
+          if (lane == 0) report(P.err, P.host_err, kErrTimeout);
           wait_tile();
           return;
         }
@@ -288,7 +288,7 @@ __device__ __forceinline__ void sweep_unit(const S& s, const SweepParams& P, int
       bad |= want[j] && y[j] >= n32;
       want[j] = want[j] && y[j] < n32;
     }
-    if (__any_sync(kFull, bad) && bad) atomicOr(P.err, kErrBadId);
+    if (__any_sync(kFull, bad) && bad) report(P.err, P.host_err, kErrBadId);
     uint32_t ry[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
     for (int j = 0; j < 4; ++j)
@@ -322,7 +322,7 @@ __device__ __forceinline__ void sweep_unit(const S& s, const SweepParams& P, int
     pos = cend;
   }
   if (kTile && pending && !wait_tile()) {   // the tile is reused by the next unit
-    if (lane == 0) atomicOr(P.err, kErrTimeout);
+    if (lane == 0) report(P.err, P.host_err, kErrTimeout);
     wait_tile();
   }
 }
@@ -424,7 +424,7 @@ __device__ __forceinline__ void serial_rows(const S& s, const SweepParams& P, ui
           if ((int)lane == first) {
             cand &= cand - 1u;
             if (yv >= n32) {
-              atomicOr(P.err, kErrBadId);
+              report(P.err, P.host_err, kErrBadId);
             } else {
               got = resolve_edge(s, xv, yv, s.raw(xv), s.raw(yv), P) ? 1u : 0u;
               got |= ld_relaxed(P.err) & kErrTimeout ? 2u : 0u;
