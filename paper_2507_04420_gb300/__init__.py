@@ -12,6 +12,7 @@ an unmatched vertex reads as -1 (0xFFFFFFFF).
 """
 from __future__ import annotations
 
+import array
 import collections
 import contextlib
 import ctypes
@@ -338,21 +339,30 @@ class Multi:
 
     @staticmethod
     def _descs(graphs, allow_host: bool = False):
-        arr = (GraphDesc * max(1, len(graphs)))()
-        for i, (off, nb, mate) in enumerate(graphs):
-            if allow_host and not off.is_cuda:
-                _need_pinned(off, "offsets", (torch.int64,))
-                _need_pinned(nb, "nbrs", _U32)
-            else:
-                _need(off, "offsets", (torch.int64,))
-                _need(nb, "nbrs", _U32)
-            _need(mate, "mate", _U32)
-            arr[i].n = off.numel() - 1
-            arr[i].nnz = nb.numel()
-            arr[i].offsets = device_address(off)
-            arr[i].nbrs = device_address(nb) if nb.numel() else None
-            arr[i].mate = mate.data_ptr() if mate.numel() else None
-        return arr
+        # one flat array of the descriptors' five words: filled field by field,
+        # ctypes structs cost more host time than a launch of small graphs takes
+        words = array.array("Q")
+        for off, nb, mate in graphs:
+            try:
+                plain = (off.is_cuda and nb.is_cuda and mate.is_cuda and off.dtype is torch.int64 and nb.dtype in _U32
+                         and mate.dtype in _U32 and off.is_contiguous() and nb.is_contiguous() and mate.is_contiguous())
+            except AttributeError:  # not tensors: refused below
+                plain = False
+            if not plain:
+                if allow_host and not off.is_cuda:
+                    _need_pinned(off, "offsets", (torch.int64,))
+                    _need_pinned(nb, "nbrs", _U32)
+                else:
+                    _need(off, "offsets", (torch.int64,))
+                    _need(nb, "nbrs", _U32)
+                _need(mate, "mate", _U32)
+            nnz, n = nb.numel(), off.numel() - 1 & 0xFFFFFFFFFFFFFFFF  # no row ends: refused by the call
+            words.extend((n, nnz, off.data_ptr() if plain else device_address(off),
+                          0 if nnz == 0 else nb.data_ptr() if plain else device_address(nb),
+                          mate.data_ptr() if mate.numel() else 0))
+        if not words:
+            return (GraphDesc * 1)()
+        return (GraphDesc * (len(words) // 5)).from_buffer(words)
 
     def run_descs(self, arr, count: int, stream=None, opts: Optional[Options] = None, **kw):
         """mm_skipper_multi over a GraphDesc array the caller filled (device addresses)."""

@@ -76,18 +76,25 @@ __global__ void multi_prepare_kernel(MultiParams M) {
   const uint64_t tid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const uint64_t nthreads = (uint64_t)gridDim.x * blockDim.x;
   const uint64_t G = M.num_graphs;
-  // every vertex ACC (Algorithm 1 lines 3-4), mate unmatched: 16 vertices a thread
+  // every vertex ACC (Algorithm 1 lines 3-4), mate unmatched: a warp fills runs
+  // of kFillRun vertices, graph by graph, one search a run
+  constexpr uint64_t kFillRun = 1024;
   const uint64_t V = M.vbase[G];
-  for (uint64_t c = tid; c * 16 < V; c += nthreads) {
-    const uint64_t v0 = c * 16;
-    uint64_t g = find_graph(M.vbase, G, v0);
-    for (uint64_t v = v0; v < v0 + 16 && v < V; ++v) {
-      while (v >= M.vbase[g + 1]) ++g;
-      M.desc[g].mate[v - M.vbase[g]] = kNone;  // = the word state ACC
+  const unsigned lane = threadIdx.x & 31u;
+  for (uint64_t v0 = (tid >> 5) * kFillRun; v0 < V; v0 += (nthreads >> 5) * kFillRun) {
+    const uint64_t v1 = v0 + kFillRun < V ? v0 + kFillRun : V;
+    uint64_t g = warp_last_at_or_below(M.vbase, G, v0, lane);
+    for (uint64_t v = v0; v < v1; ++g) {
+      const uint64_t first = __ldg(M.vbase + g), last = __ldg(M.vbase + g + 1);
+      const uint64_t stop = last < v1 ? last : v1;
+      uint32_t* const mate = M.desc[g].mate;
+      for (uint64_t i = v + lane; i < stop; i += 32) mate[i - first] = kNone;  // = the word state ACC
+      v = stop;
     }
   }
   if (!kWord)
-    for (uint64_t i = tid; i < M.sbase[G]; i += nthreads) M.state_pool[i] = 0u;
+    for (uint64_t i = tid; i < (M.sbase[G] + 3) / 4; i += nthreads)  // the pool holds whole quads
+      reinterpret_cast<uint4*>(M.state_pool)[i] = make_uint4(0u, 0u, 0u, 0u);
   // merge-path units of every graph
   for (uint64_t u = tid; u < M.units; u += nthreads) {
     const uint64_t g = find_graph(M.ubase, G, u);
@@ -433,7 +440,7 @@ mm_status mm_skipper_multi(mm_multi* m, uint64_t num_graphs, const mm_graph_desc
   if ((st = stage_tables(&m->sweep, num_graphs, h_descs, grain, (int)bits, s, &L)) != MM_OK) return st;
   MTRY(grow(&m->sweep.part, &m->sweep.part_cap, 2 * (L.units + 1), s));
   MTRY(grow(&m->sweep.gid, &m->sweep.gid_cap, L.units + 1, s));
-  if (!word) MTRY(grow(&m->pool, &m->pool_cap, L.total_words + 1, s));
+  if (!word) MTRY(grow(&m->pool, &m->pool_cap, L.total_words + 4, s));
   MultiParams M = params(m, m->sweep, num_graphs, L, grain, o->spin_limit ? o->spin_limit : (1ull << 20));
   M.disperse = disperse ? 1u : 0u;
   m->h_err[1] = 0;  // a call that waits has its kernels report here
