@@ -47,8 +47,24 @@ struct ChipState {
   __device__ static __forceinline__ uint32_t shift(uint32_t v) { return (v % kPerWord) * kBits; }
   __device__ __forceinline__ uint32_t raw(uint32_t v) const { return lds(at(v)); }
   __device__ __forceinline__ uint32_t peek(uint32_t v) const { return lds(at(v)); }
-  __device__ static __forceinline__ bool matched(uint32_t raw, uint32_t v) {
-    return ((raw >> shift(v)) & kMask) == kMchd;
+  __device__ static __forceinline__ bool matched(uint32_t raw, uint32_t v) { return (raw >> shift(v)) & kMchd; }
+  __device__ __forceinline__ uint32_t take(uint32_t v) const {
+    uint32_t old;
+    asm volatile("atom.relaxed.cta.shared::cta.or.b32 %0, [%1], %2;"
+                 : "=r"(old)
+                 : "r"(at(v)), "r"(kRsvd << shift(v))
+                 : "memory");
+    return (old >> shift(v)) & kMask;
+  }
+  __device__ __forceinline__ void put_back(uint32_t v, uint32_t was) const {
+    if (!(was & kRsvd))
+      asm volatile("red.relaxed.cta.shared::cta.and.b32 [%0], %1;" ::"r"(at(v)), "r"(~(kRsvd << shift(v))) : "memory");
+  }
+  __device__ __forceinline__ void commit_both(uint32_t u, uint32_t v) const {
+    mate[u] = v;
+    mate[v] = u;
+    flip(u, kRsvd ^ kMchd);
+    flip(v, kRsvd ^ kMchd);
   }
   __device__ __forceinline__ bool cas(uint32_t v, uint32_t expect, uint32_t desired, uint32_t& cur,
                                       const SweepParams& P) const {
