@@ -224,7 +224,7 @@ __global__ void batch_serial_kernel(BatchParams B) {
   if (g >= B.num_graphs) return;
   const SweepParams P = graph_view<kLocal, kWord>(B, g);
   if (kLocal)
-    serial_rows(S(P), P, 0, P.n, threadIdx.x & 31u);
+    serial_graph<S>(P, threadIdx.x & 31u);
   else
     serial_rows(S(P), P, (uint64_t)B.vbase[g], (uint64_t)B.vbase[g + 1], threadIdx.x & 31u);
 }

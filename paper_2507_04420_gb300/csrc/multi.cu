@@ -143,7 +143,7 @@ __global__ void multi_serial_kernel(MultiParams M) {
   const uint64_t g = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;  // one warp a graph
   if (g >= M.num_graphs) return;
   const SweepParams P = view(M, g, kWord);
-  serial_rows(S(P), P, 0, P.n, threadIdx.x & 31u);
+  serial_graph<S>(P, threadIdx.x & 31u);
 }
 
 __device__ __forceinline__ void group_add(unsigned long long* c, unsigned peers, uint32_t v) {

@@ -260,6 +260,7 @@ struct Waiter {
 template <int kBits>
 struct PackedState {
   static constexpr bool kNear = false;
+  static constexpr bool kAlone = false;
   static constexpr uint32_t kPerWord = 32u / kBits;
   static constexpr uint32_t kMask = (1u << kBits) - 1u;
   uint32_t* words;
@@ -365,6 +366,7 @@ __host__ __device__ __forceinline__ uint64_t packed_words(uint64_t n, int bits) 
 
 struct WordState {
   static constexpr bool kNear = false;
+  static constexpr bool kAlone = false;
   static constexpr uint32_t kPerWord = 1;
   uint32_t* words;
   __device__ explicit WordState(const SweepParams& P) : words(P.state) {}
