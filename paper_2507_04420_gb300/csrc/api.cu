@@ -282,6 +282,12 @@ SweepParams make_params(mm_graph* g, const Resolved& r, uint32_t* d_mate) {
   P.tile = r.stage && !r.serial && !r.word && !g->host_mapped && aligned16;
   // the 32-register instance exists for the plain and symmetric sweeps only
   P.lean = r.lean && !r.serial && !r.stats && !P.sel && !P.tile;
+  // Fewer than 5 entries a row: lattices, quad meshes, road networks.  Calls, in
+  // us, without / with the second visits: a 4096 x 4096 grid, bytes 942 / 822, 2
+  // bits 1162 / 826, words 1284 / 763, a 300 x 700 grid 105 / 76; an Erdos-Renyi
+  // graph of 4 entries a row, which has no locality, 720 / 744.  Above, R-MAT 27
+  // 4822 / 5135, uniform of 20 entries a row 1515 / 1625.
+  P.mesh = P.lean && g->nnz < 5 * g->n;
   P.disperse = r.disperse ? 1u : 0u;
   return P;
 }

@@ -71,6 +71,8 @@ struct SweepParams {
   // 1: the plain or symmetric instance compiled for 32 registers a thread
   // (64 warps per SM) instead of 40 (48 warps per SM)
   uint32_t lean;
+  // 1: the lean instance that visits a chunk naming its own rows twice (kMesh)
+  uint32_t mesh;
   // 1: work units handed out in dispersed runs (one run per warp of the grid)
   uint32_t disperse;
 };

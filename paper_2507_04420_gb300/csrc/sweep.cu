@@ -85,7 +85,7 @@ __global__ void prepare_kernel(SweepParams P, uint64_t* graph_pairs, uint64_t nu
 // a few more spills), which hides more memory latency where the state array
 // stays in L2.
 template <class S, bool kStats = false, bool kSym = false, bool kSel = false, bool kTile = false,
-          bool kLean = false>
+          bool kLean = false, bool kMesh = false>
 __global__ void __launch_bounds__(512, kLean ? 4 : 3) sweep_kernel(SweepParams P) {
   const unsigned lane = threadIdx.x & 31u;
   const S s(P);
@@ -109,7 +109,7 @@ __global__ void __launch_bounds__(512, kLean ? 4 : 3) sweep_kernel(SweepParams P
     const int64_t e_begin = P.part[2 * w + 1];
     const int64_t e_end = P.part[2 * w + 3];
     if (e_begin < e_end)
-      sweep_unit<S, kStats, kSym, kSel, kTile>(s, P, row0, e_begin, e_end, lane, pol, &phase);
+      sweep_unit<S, kStats, kSym, kSel, kTile, kMesh>(s, P, row0, e_begin, e_end, lane, pol, &phase);
     if ((c & 15) == 0) {  // stop handing out work once an error is recorded
       uint32_t e = 0;
       if (lane == 0) e = ld_relaxed(P.err);
@@ -221,12 +221,14 @@ cudaError_t launch_sweep(const SweepParams& P, int bits, int grid, int block, cu
     SKP_DISPATCH_STATE(bits, L);
 #undef L
   } else if (P.sym) {
-#define L(S, B) (P.lean ? (sweep_kernel<S, false, true, false, false, true><<<grid, block, 0, s>>>(P), 0) \
+#define L(S, B) (P.mesh ? (sweep_kernel<S, false, true, false, false, true, true><<<grid, block, 0, s>>>(P), 0) \
+                 : P.lean ? (sweep_kernel<S, false, true, false, false, true><<<grid, block, 0, s>>>(P), 0) \
                         : (sweep_kernel<S, false, true><<<grid, block, 0, s>>>(P), 0))
     SKP_DISPATCH_STATE(bits, L);
 #undef L
   } else {
-#define L(S, B) (P.lean ? (sweep_kernel<S, false, false, false, false, true><<<grid, block, 0, s>>>(P), 0) \
+#define L(S, B) (P.mesh ? (sweep_kernel<S, false, false, false, false, true, true><<<grid, block, 0, s>>>(P), 0) \
+                 : P.lean ? (sweep_kernel<S, false, false, false, false, true><<<grid, block, 0, s>>>(P), 0) \
                         : (sweep_kernel<S><<<grid, block, 0, s>>>(P), 0))
     SKP_DISPATCH_STATE(bits, L);
 #undef L

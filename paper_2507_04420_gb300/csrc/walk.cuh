@@ -108,6 +108,12 @@ __device__ __forceinline__ void init_window_tile(unsigned lane) {
 // of the row at the head of each chunk is re-read alongside, so a long row
 // matched by another warp is left after at most one more chunk.
 //
+// kMesh (graphs of few entries a row, most of them lattices, meshes and road
+// networks): where ids have locality the rows of a window name each other, as x
+// names x - 1 all along it; tried at once, each holds what the next one waits
+// for.  So a chunk that names rows of its own window is visited twice, the odd
+// rows waiting for the second visit.
+//
 // kTile: windows come from the warp's shared-memory tile (WindowTile above).
 //
 // kSel (selective id loads): a lane loads its quad only after the row search,
@@ -116,7 +122,7 @@ __device__ __forceinline__ void init_window_tile(unsigned lane) {
 // overlaps the search; the selective walk moves fewer bytes (on R-MAT, well
 // under half the quads of a chunk are in rows not known matched), which pays
 // where the bytes cross the host link.
-template <class S, bool kStats = false, bool kSym = false, bool kSel = false, bool kTile = false>
+template <class S, bool kStats = false, bool kSym = false, bool kSel = false, bool kTile = false, bool kMesh = false>
 __device__ __forceinline__ void sweep_unit(const S& s, const SweepParams& P, int64_t row0,
                                            const int64_t e_begin, const int64_t e_end,
                                            const unsigned lane, const uint64_t pol_stream,
@@ -137,6 +143,7 @@ __device__ __forceinline__ void sweep_unit(const S& s, const SweepParams& P, int
   uint32_t my_st;
   unsigned mchd;
   int pos = 0;
+  bool again = false;                           // second visit to a chunk (kMesh)
   bool pending = false;                         // a copy of the next window's tile is in flight
   auto tile = [&]() { return &g_window_tiles[threadIdx.x >> 5]; };
   auto t_s = [&](int64_t w) { return (w + 1) & ~(int64_t)1; };
@@ -175,12 +182,17 @@ __device__ __forceinline__ void sweep_unit(const S& s, const SweepParams& P, int
     issue_next(wbase + 32);
   }
   while (pos < ue) {
+    if (kMesh && again) {  // what the first visit left open
+      if (wbase + lane < (int64_t)P.n) my_st = s.peek((uint32_t)wbase + lane);
+      mchd |= __ballot_sync(kFull, S::matched(my_st, (uint32_t)wbase + lane));
+    }
     // rows of the window with entries at or after pos that are not known matched
     const unsigned open = __ballot_sync(kFull, my_end > pos) & ~mchd;
     if (open == 0u) {  // the window is exhausted: continue after its last row
       const int win_end = __shfl_sync(kFull, my_end, 31);
       if (win_end >= ue) break;
       if (win_end > pos) pos = win_end;
+      if (kMesh) again = false;
       wbase += 32;
       const int64_t r = wbase + lane;
       const bool in = r < (int64_t)P.n;
@@ -299,6 +311,18 @@ __device__ __forceinline__ void sweep_unit(const S& s, const SweepParams& P, int
     for (int j = 0; j < 4; ++j)
       if (want[j] && !S::matched(ry[j], y[j])) cand |= 1u << j;
 
+    if (kMesh) {
+      bool near = false;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) near |= (cand >> j & 1u) && y[j] - wb32 < 32u;
+      again = !again && __any_sync(kFull, near);
+      if (again) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (k[j] & 1) cand &= ~(1u << j);
+      }
+    }
+
     // resolve candidates: per row, one lane at a time
     for (;;) {
       const bool have = cand != 0u;
@@ -320,7 +344,7 @@ __device__ __forceinline__ void sweep_unit(const S& s, const SweepParams& P, int
       for (int jj = 0; jj < 4; ++jj)
         if (done >> (k[jj] & 31) & 1u) cand &= ~(1u << jj);
     }
-    pos = cend;
+    if (!kMesh || !again) pos = cend;
   }
   if (kTile && pending && !wait_tile()) {   // the tile is reused by the next unit
     if (lane == 0) report(P.err, P.host_err, kErrTimeout);
