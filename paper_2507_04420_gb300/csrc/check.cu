@@ -86,7 +86,7 @@ __global__ void __launch_bounds__(256, kCheckBlocks) check_csr_kernel(CheckView 
 // the queued rows of unmatched vertices, each spread over the grid
 __global__ void check_csr_long_kernel(CheckView V, LongRows queue, unsigned long long* __restrict__ c,
                                       unsigned long long* __restrict__ host) {
-  const unsigned long long rows = *queue.count;
+  const unsigned long long rows = queue.size();
   for (unsigned long long i = 0; i < rows; ++i)
     check_long_row(V, (uint32_t)queue.items[i], c, threadIdx.x & 31u);
   publish_counters<true>(c, host);
@@ -347,7 +347,7 @@ cudaError_t launch_validate(uint64_t n, uint64_t nnz, const int64_t* offsets, co
     validate_pairs_kernel<<<grid, 256, 0, s>>>(n, mate, pairs, count, cs.seen_bits, cs.counters);
   }
   const CheckView V{offsets, nbrs, mate, n, nnz};
-  const LongRows queue{cs.counters + kCkLong, cs.long_rows};
+  const LongRows queue{cs.counters + kCkLong, cs.long_rows, long_row_cap(nnz)};
   check_csr_kernel<<<check_grid(n, sms), 256, 0, s>>>(V, queue, cs.counters, cs.host);
   return cudaGetLastError();
 }
@@ -357,7 +357,8 @@ bool validate_needs_long(const CheckScratch& cs) { return cs.host[kCkLong] != 0;
 cudaError_t launch_validate_long(uint64_t n, uint64_t nnz, const int64_t* offsets, const uint32_t* nbrs,
                                  const uint32_t* mate, const CheckScratch& cs, int sms, cudaStream_t s) {
   check_csr_long_kernel<<<sms * 4, 256, 0, s>>>(CheckView{offsets, nbrs, mate, n, nnz},
-                                                LongRows{cs.counters + kCkLong, cs.long_rows}, cs.counters, cs.host);
+                                                LongRows{cs.counters + kCkLong, cs.long_rows, long_row_cap(nnz)},
+                                                cs.counters, cs.host);
   return cudaGetLastError();
 }
 

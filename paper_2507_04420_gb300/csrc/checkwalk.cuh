@@ -59,10 +59,19 @@ struct Visit {
   unsigned long long first_unc = ~0ull;
 };
 
-// rows of unmatched vertices left to the second kernel: graph << 32 | vertex
+// rows of unmatched vertices left to the second kernel: graph << 32 | vertex.
+// cap counts the rows that can be so long when none overlap; row ends that were
+// never checked may overlap, and what does not fit is read at once.
 struct LongRows {
   unsigned long long* count;
   uint64_t* items;
+  uint64_t cap;
+  __device__ __forceinline__ bool push(uint64_t item) const {
+    const unsigned long long at = atomicAdd(count, 1ull);
+    if (at < cap) items[at] = item;
+    return at < cap;
+  }
+  __device__ __forceinline__ unsigned long long size() const { return *count < cap ? *count : cap; }
 };
 
 // last g < G with base[g] <= x (base ascending, base[0] = 0 <= x < base[G]), found by the whole warp
@@ -233,9 +242,8 @@ __device__ __forceinline__ Visit check_group(const CheckView& V, bool in, uint32
         hit = warp_row_has(nbrs, nnz, __ldg(offsets + tj), __ldg(offsets + tj + 1), tj ^ oj, lane);
       }
       if (!hit && (int)lane == j) a.bits |= kVxNonedge;
-    } else if (ej - sj > kLongRow) {
-      if ((int)lane == j) queue.items[atomicAdd(queue.count, 1ull)] = (uint64_t)graph << 32 | v;
-    } else {
+    } else if (ej - sj <= kLongRow ||
+               !__shfl_sync(kFull, (int)lane == j && queue.push((uint64_t)graph << 32 | v) ? 1 : 0, j)) {
       const uint32_t xj = __shfl_sync(kFull, v, j);
       const uint32_t* mate = kOne ? V.mate : shfl_ptr(V.mate, j);
       const uint64_t n = kOne ? V.n : __shfl_sync(kFull, V.n, j);

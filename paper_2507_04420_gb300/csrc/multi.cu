@@ -212,7 +212,7 @@ __global__ void __launch_bounds__(256, kCheckBlocks) multi_check_kernel(MultiPar
 }
 
 __global__ void multi_check_long_kernel(MultiParams M, LongRows queue) {
-  const unsigned long long rows = *queue.count;
+  const unsigned long long rows = queue.size();
   for (unsigned long long i = 0; i < rows; ++i) {
     const uint64_t item = queue.items[i];
     check_long_row(multi_check_view(M, item >> 32), (uint32_t)item, M.counters + (item >> 32) * kCkCount,
@@ -518,7 +518,7 @@ mm_status mm_validate_multi_async(mm_multi* m, uint64_t num_graphs, const mm_gra
     m->h_counters_cap = cap;
   }
   const MultiParams M = params(m, m->check, num_graphs, L, (uint64_t)kLongRow, 1);
-  const LongRows queue{m->counters + words, reinterpret_cast<uint64_t*>(m->check.part)};
+  const LongRows queue{m->counters + words, reinterpret_cast<uint64_t*>(m->check.part), L.long_rows};
   MTRY(cudaMemsetAsync(m->counters, 0, (words + 1) * sizeof(unsigned long long), s));
   if (L.total_vertices) {
     multi_check_kernel<<<check_grid(L.total_vertices, m->num_sms), 256, 0, s>>>(M, queue);
