@@ -428,7 +428,7 @@ __device__ __forceinline__ bool resolve_edge(const S& s, uint32_t x, uint32_t y,
   Waiter<S::kNear> wt;
   uint32_t cnf = 0;                          // conflicts on this entry (kStats only)
   bool result = false;
-  if constexpr (!kStats) {
+  if (!kStats && (S::kPerWord > 1 || P.lean)) {
     // The first attempt takes both endpoints at once: where it succeeds (99% of
     // the attempts on uniform graphs) the edge costs one round trip instead of
     // two in a row, and no retries when a neighbouring field changes under a CAS,
@@ -439,6 +439,8 @@ __device__ __forceinline__ bool resolve_edge(const S& s, uint32_t x, uint32_t y,
     // vertices in 2 bits 2280 / 1510, R-MAT 27 in bytes 5190 / 4817, R-MAT 18
     // 186 / 145, the 4096-graph batch 1373 / 1145, a 4096 x 4096 grid 1122 / 950.
     // (One atomic for both fields when they share a word: no faster anywhere.)
+    // Word states are taken so only where they stay in L2: in DRAM the second
+    // store to v's sector costs more, R-MAT 27 6.04 -> 6.17 ms a sweep.
     if (S::matched(ru, u) || S::matched(rv, v)) return S::matched(x_low ? ru : rv, x);  // line 10
     const uint32_t fu = s.take(u), fv = s.take(v);
     if ((fu | fv) == kAcc) {
