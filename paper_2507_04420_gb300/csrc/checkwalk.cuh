@@ -48,6 +48,7 @@ struct CheckView {
   const uint32_t* nbrs;
   const uint32_t* mate;
   uint64_t n, nnz;
+  __device__ __forceinline__ int64_t end(uint64_t v) const { return row_end(offsets, v, nnz); }
 };
 
 // what one visit found: the vertex's bits, and the uncovered entries this lane met
@@ -167,8 +168,8 @@ __device__ __forceinline__ VertexRow load_vertex(const CheckView& V, bool in, ui
   VertexRow r;
   if (in) {
     r.m = __ldg(V.mate + v);
-    r.s = __ldg(V.offsets + v);
-    r.e = __ldg(V.offsets + v + 1);
+    r.s = V.end(v);
+    r.e = V.end((uint64_t)v + 1);
   }
   return r;
 }
@@ -190,7 +191,7 @@ __device__ __forceinline__ Visit check_group(const CheckView& V, bool in, uint32
       a.bits = kVxMatched | (sym ? kVxBothEnds | (v < m ? kVxPair : 0u) : kVxAsym);
       find = !sym || v < m;
       if (find) {
-        const int64_t s2 = __ldg(V.offsets + m), e2 = __ldg(V.offsets + m + 1);
+        const int64_t s2 = V.end(m), e2 = V.end((uint64_t)m + 1);
         if (e2 - s2 < e - s) {             // the shorter row first
           s = s2;
           e = e2;
@@ -219,8 +220,8 @@ __device__ __forceinline__ Visit check_group(const CheckView& V, bool in, uint32
     if (s < e) continue;
     if (find && again) {
       again = false;
-      s = __ldg(V.offsets + t);
-      e = __ldg(V.offsets + t + 1);
+      s = V.end(t);
+      e = V.end((uint64_t)t + 1);
       t ^= other;
     } else {
       todo = false;
@@ -239,7 +240,7 @@ __device__ __forceinline__ Visit check_group(const CheckView& V, bool in, uint32
       bool hit = warp_row_has(nbrs, nnz, sj, ej, tj, lane);
       if (!hit && __shfl_sync(kFull, again ? 1 : 0, j)) {
         const int64_t* offsets = kOne ? V.offsets : shfl_ptr(V.offsets, j);
-        hit = warp_row_has(nbrs, nnz, __ldg(offsets + tj), __ldg(offsets + tj + 1), tj ^ oj, lane);
+        hit = warp_row_has(nbrs, nnz, row_end(offsets, tj, nnz), row_end(offsets, (uint64_t)tj + 1, nnz), tj ^ oj, lane);
       }
       if (!hit && (int)lane == j) a.bits |= kVxNonedge;
     } else if (ej - sj <= kLongRow ||
@@ -298,7 +299,7 @@ __device__ __forceinline__ void add_faults(unsigned long long* c, const Visit& a
 // One queued row, spread over the whole grid.
 __device__ __forceinline__ void check_long_row(const CheckView& V, uint32_t x, unsigned long long* c,
                                                unsigned lane) {
-  const int64_t s = __ldg(V.offsets + x), e = __ldg(V.offsets + x + 1);
+  const int64_t s = V.end(x), e = V.end((uint64_t)x + 1);
   const int64_t step = 4 * (int64_t)gridDim.x * blockDim.x;
   Visit a;  // an entry in 4 * step: 32 bits hold a lane's share
   for (int64_t q = (s & ~(int64_t)3) + 4 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x); q < e; q += step)

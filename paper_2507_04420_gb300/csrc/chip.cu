@@ -125,15 +125,13 @@ __device__ __forceinline__ void chip_graph(const SweepParams& P, ChipShared& sh,
   __syncthreads();
   const S s{smem_u32(g_chip_words), P.mate};
   const uint32_t windows = (n + 31) / 32;
-  // row ends of a CSR that was not checked still stay inside the entries
-  auto clamp = [&](int64_t e) { return e < 0 ? (int64_t)0 : e > (int64_t)P.nnz ? (int64_t)P.nnz : e; };
   for (;;) {
     uint32_t w = 0;
     if (lane == 0) w = atomicAdd(&sh.next, 1u);
     w = __shfl_sync(kFull, w, 0);
     if (w >= windows) break;
     const uint32_t r0 = 32 * w, r1 = r0 + 32 < n ? r0 + 32 : n;
-    const int64_t e0 = clamp(__ldg(P.offsets + r0)), e1 = clamp(__ldg(P.offsets + r1));
+    const int64_t e0 = row_end(P.offsets, r0, P.nnz), e1 = row_end(P.offsets, r1, P.nnz);
     if (e1 - e0 > kLongWindow) {
       uint32_t k = 0;
       if (lane == 0) k = atomicAdd(&sh.nlong, 1u);
@@ -149,8 +147,8 @@ __device__ __forceinline__ void chip_graph(const SweepParams& P, ChipShared& sh,
   const uint32_t nlong = sh.nlong < kMaxLong ? sh.nlong : kMaxLong;
   for (uint32_t k = 0; k < nlong; ++k) {
     const uint32_t r0 = 32 * sh.longs[k], r1 = r0 + 32 < n ? r0 + 32 : n;
-    const int64_t e1 = clamp(__ldg(P.offsets + r1));
-    for (int64_t e = clamp(__ldg(P.offsets + r0)) + kPiece * (threadIdx.x >> 5); e < e1; e += kPiece * (blockDim.x >> 5))
+    const int64_t e1 = row_end(P.offsets, r1, P.nnz);
+    for (int64_t e = row_end(P.offsets, r0, P.nnz) + kPiece * (threadIdx.x >> 5); e < e1; e += kPiece * (blockDim.x >> 5))
       sweep_unit<S, false, kSym>(s, P, r0, e, e + kPiece < e1 ? e + kPiece : e1, lane, pol);
   }
   if (nlong) __syncthreads();
