@@ -260,12 +260,15 @@ __global__ void batch_pairs_kernel(BatchParams B) {
 // one verdict for all member graphs; the vertex and entry indices it names are
 // the batch's.  (With global ids a batch is one CSR: launch_validate.)  A warp
 // takes runs of kCheckRun * 32 vertices, so that one search of vbase serves a
-// run and a lane then only steps on to the next graph. ----
+// run and a lane then only steps on to the next graph.  vbase is read where it
+// lies and never checked: a graph's vertices end with the batch's, and a vertex
+// before its graph's first is left out. ----
 constexpr uint64_t kCheckRun = 4;
 
 __device__ __forceinline__ CheckView batch_check_view(const BatchParams& B, uint64_t g) {
-  const int64_t vb = __ldg(B.vbase + g);
-  return CheckView{B.P.offsets + vb, B.P.nbrs, B.P.mate + vb, (uint64_t)(__ldg(B.vbase + g + 1) - vb), B.P.nnz};
+  const uint64_t vb = (uint64_t)__ldg(B.vbase + g), ve = (uint64_t)__ldg(B.vbase + g + 1);
+  const uint64_t end = ve < B.P.n ? ve : B.P.n;
+  return CheckView{B.P.offsets + vb, B.P.nbrs, B.P.mate + vb, end > vb ? end - vb : 0, B.P.nnz};
 }
 
 __global__ void __launch_bounds__(256, kCheckBlocks) batch_check_kernel(BatchParams B, LongRows queue,
@@ -280,10 +283,10 @@ __global__ void __launch_bounds__(256, kCheckBlocks) batch_check_kernel(BatchPar
     uint64_t g = warp_last_at_or_below(B.vbase, G, w0, lane);
     for (uint64_t v0 = w0; v0 < w0 + 32 * kCheckRun && v0 < N; v0 += 32) {
       const uint64_t i = v0 + lane;
-      const bool in = i < N;
-      while (in && (int64_t)i >= __ldg(B.vbase + g + 1)) ++g;
+      while (i < N && g + 1 < G && i >= (uint64_t)__ldg(B.vbase + g + 1)) ++g;
       const CheckView V = batch_check_view(B, g);
-      const uint64_t vb = (uint64_t)(V.mate - B.P.mate);
+      const uint64_t vb = (uint64_t)__ldg(B.vbase + g);
+      const bool in = i < N && i >= vb;
       const uint32_t v = (uint32_t)(i - vb);
       const Visit a = check_group<false>(V, in, v, load_vertex(V, in, v), (uint32_t)g, lane, queue);
       matched += __popc(__ballot_sync(kFull, a.bits & kVxMatched));

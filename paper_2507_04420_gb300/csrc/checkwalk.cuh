@@ -75,14 +75,15 @@ struct LongRows {
   __device__ __forceinline__ unsigned long long size() const { return *count < cap ? *count : cap; }
 };
 
-// last g < G with base[g] <= x (base ascending, base[0] = 0 <= x < base[G]), found by the whole warp
+// last g < G with base[g] <= x (base ascending, base[0] = 0 <= x < base[G]), found by the whole warp;
+// some g < G whatever base holds
 template <class T>
 __device__ __forceinline__ uint64_t warp_last_at_or_below(const T* base, uint64_t G, uint64_t x, unsigned lane) {
   uint64_t lo = 0, hi = G;
   while (hi - lo > 1) {
     const uint64_t step = (hi - lo + 31) / 32, at = lo + lane * step;
     const unsigned below = __ballot_sync(kFull, at < hi && (uint64_t)__ldg(base + at) <= x);
-    lo += (uint64_t)(__popc(below) - 1) * step;
+    lo += (uint64_t)(below ? __popc(below) - 1 : 0) * step;
     hi = lo + step < hi ? lo + step : hi;
   }
   return lo;
