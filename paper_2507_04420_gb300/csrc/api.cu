@@ -282,6 +282,7 @@ SweepParams make_params(mm_graph* g, const Resolved& r, uint32_t* d_mate) {
   P.tile = r.stage && !r.serial && !r.word && !g->host_mapped && aligned16;
   // the 32-register instance exists for the plain and symmetric sweeps only
   P.lean = r.lean && !r.serial && !r.stats && !P.sel && !P.tile;
+  P.both = P.lean && P.units <= (uint64_t)g->num_sms * 64;
   // Fewer than 5 entries a row: lattices, quad meshes, road networks.  Calls, in
   // us, without / with the second visits: a 4096 x 4096 grid, bytes 942 / 822, 2
   // bits 1162 / 826, words 1284 / 763, a 300 x 700 grid 105 / 76; an Erdos-Renyi

@@ -12,7 +12,7 @@
 //     that is retried when only a neighbouring field changed.  The holder-only
 //     transitions RSVD->MCHD and RSVD->ACC (Algorithm 1 lines 15 and 18, plain
 //     stores in the paper) become one atomic XOR on the word, which cannot
-//     disturb the neighbouring fields.  A first attempt on an edge sets the RSVD
+//     disturb the neighbouring fields.  The first attempt on an edge sets the RSVD
 //     bits of both its vertices with atomic ORs (resolve_edge); on a matched
 //     vertex that bit is a stray one until it is cleared, and the field still
 //     reads as matched.  The statistics instances make the ordered transitions
@@ -71,6 +71,8 @@ struct SweepParams {
   // 1: the plain or symmetric instance compiled for 32 registers a thread
   // (64 warps per SM) instead of 40 (48 warps per SM)
   uint32_t lean;
+  // 1: word states, too: the first attempt takes both endpoints at once
+  uint32_t both;
   // 1: the lean instance that visits a chunk naming its own rows twice (kMesh)
   uint32_t mesh;
   // 1: work units handed out in dispersed runs (one run per warp of the grid)
@@ -435,7 +437,7 @@ __device__ __forceinline__ bool resolve_edge(const S& s, uint32_t x, uint32_t y,
   Waiter<S::kNear> wt;
   uint32_t cnf = 0;                          // conflicts on this entry (kStats only)
   bool result = false;
-  if (!kStats && (S::kPerWord > 1 || P.lean)) {
+  if (!kStats && (S::kPerWord > 1 || P.both)) {
     // The first attempt takes both endpoints at once: where it succeeds (99% of
     // the attempts on uniform graphs) the edge costs one round trip instead of
     // two in a row, and no retries when a neighbouring field changes under a CAS,
@@ -446,8 +448,14 @@ __device__ __forceinline__ bool resolve_edge(const S& s, uint32_t x, uint32_t y,
     // vertices in 2 bits 2280 / 1510, R-MAT 27 in bytes 5190 / 4817, R-MAT 18
     // 186 / 145, the 4096-graph batch 1373 / 1145, a 4096 x 4096 grid 1122 / 950.
     // (One atomic for both fields when they share a word: no faster anywhere.)
-    // Word states are taken so only where they stay in L2: in DRAM the second
-    // store to v's sector costs more, R-MAT 27 6.04 -> 6.17 ms a sweep.
+    // Words share nothing, so a CAS on one fails only to another attempt on the
+    // vertex, and claiming v is its mate entry's only store: taken both at once they
+    // cost a store more, which pays where the call waits on its attempts one after
+    // the other -- every unit has a warp (P.both) -- and costs uniform graphs where
+    // many are in flight.  Calls, ordered / both: uniform, 100 K vertices of 8
+    // entries 61 / 58 (8192 items a unit 191 / 171), 16 M of 4 entries 567 / 586, 2 M
+    // of 16 196 / 210, symmetric 160 / 183; R-MAT 14 85 / 68, 27 6.04 / 6.17 ms a sweep,
+    // between them 20 would gain (125 / 112) and 22 not (208 / 210).
     if (S::matched(ru, u) || S::matched(rv, v)) return S::matched(x_low ? ru : rv, x);  // line 10
     const uint32_t fu = s.take(u), fv = s.take(v);
     if ((fu | fv) == kAcc) {
