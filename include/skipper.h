@@ -85,10 +85,10 @@ typedef struct mm_options {
                                 when set.  0 = chosen from the graph: about two
                                 units per resident sweep warp, the nearest power
                                 of two in [512, 8192], at most 4096 where units are
-                                dispersed (2048 below 16 rows + entries a row,
-                                1024 below 8), up to 32768 for MM_HOST_MAPPED
-                                handles, whose units each start by waiting on the
-                                host link.  Batched and multi-graph calls choose
+                                dispersed by default or by request (2048 below 16
+                                rows + entries a row; 1024 below 8, in the 32-bit
+                                layout below 6), up to 32768 for MM_HOST_MAPPED handles,
+                                whose units each start by waiting on the host link.  Batched and multi-graph calls choose
                                 from all their graphs together, down to 128.
                                 mm_skipper_static takes 0 as 2048. */
     uint32_t block_threads;  /* sweep threads per block, multiple of 32, <= 512;

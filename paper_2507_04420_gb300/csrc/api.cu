@@ -150,7 +150,11 @@ struct Resolved {
 // 8192 (R-MAT 27: 4640, 4096 takes 4690).  Dispersed ones 4096 (2^26 edges of
 // factor 16: R-MAT 214, uniform 520; 8192 takes 229, 570), less where rows are
 // short: 2048 (R-MAT of edge factor 6: 343, 4096 takes 351, 1024 takes 459),
-// 1024 below 8 items a row (a 4096 x 4096 grid 804, 4096 takes 930).
+// 1024 below 8 items a row (calls, 1024 / 2048: a 4096 x 4096 grid 520 / 586), with
+// word states below 6: their attempts cost less, so that units of 1024 cost uniform
+// graphs more than they spare lattices (16 M vertices of 6 entries 673 / 616 against
+// 628 at 4096; R-MAT 24 of edge factor 3 409 / 361; grid 474 / 548, path 304 / 330;
+// uniform of 4 entries, which no count of entries tells from a lattice, 571 / 530).
 // Over the host link every unit's first window waits on the link: up to 32768.
 uint32_t grain_between(uint64_t items, uint64_t warps, uint64_t least, uint64_t most) {
   const uint64_t target = items / (2 * warps);
@@ -158,9 +162,9 @@ uint32_t grain_between(uint64_t items, uint64_t warps, uint64_t least, uint64_t 
   while (grain < most && grain * 1414 < target * 1000) grain *= 2;
   return (uint32_t)grain;
 }
-uint64_t most_grain(uint64_t rows, uint64_t items, bool disperse) {
+uint64_t most_grain(uint64_t rows, uint64_t items, bool disperse, bool word) {
   const uint64_t row = rows ? items / rows : 1;
-  return !disperse ? 8192 : row < 8 ? 1024 : row < 16 ? 2048 : 4096;
+  return !disperse ? 8192 : row < (word ? 6 : 8) ? 1024 : row < 16 ? 2048 : 4096;
 }
 }  // namespace
 
@@ -168,9 +172,9 @@ uint64_t most_grain(uint64_t rows, uint64_t items, bool disperse) {
 // is one unit's chain of windows, so short rows take units down to 128 (64
 // graphs of 100 to 10,000 edges: 58 at 256, 70 at 512; 4096 mixed graphs: 953
 // at 2048, 8192 takes 1223).
-uint32_t skp::choose_grain(uint64_t rows, uint64_t items, uint64_t warps, bool disperse) {
+uint32_t skp::choose_grain(uint64_t rows, uint64_t items, uint64_t warps, bool disperse, bool word) {
   const uint64_t row = rows ? items / rows : 1;
-  return grain_between(items, warps, row < 8 ? 128 : row < 24 ? 256 : 512, most_grain(rows, items, disperse));
+  return grain_between(items, warps, row < 8 ? 128 : row < 24 ? 256 : 512, most_grain(rows, items, disperse, word));
 }
 
 namespace {
@@ -214,8 +218,8 @@ mm_status resolve(const mm_graph* g, const mm_options* o, Resolved* r, bool batc
   if (r->grain == 0) {
     const uint64_t warps = (uint64_t)(g->num_sms > 0 ? g->num_sms : 1) * (r->lean ? 64u : 48u);
     const uint64_t items = g->coo ? g->nnz : g->n + g->nnz;
-    const uint64_t most = g->host_mapped ? 32768 : g->coo ? 8192 : most_grain(g->n, items, r->disperse);
-    r->grain = batch && !g->host_mapped ? choose_grain(g->n, items, warps, r->disperse)
+    const uint64_t most = g->host_mapped ? 32768 : g->coo ? 8192 : most_grain(g->n, items, r->disperse, r->word);
+    r->grain = batch && !g->host_mapped ? choose_grain(g->n, items, warps, r->disperse, r->word)
                                         : grain_between(items, warps, 512, most);
   }
   r->spin_limit = o->spin_limit ? o->spin_limit : kDefaultSpin;

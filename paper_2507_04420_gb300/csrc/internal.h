@@ -60,7 +60,7 @@ cudaError_t launch_validate_batch_long(const BatchParams& B, const CheckScratch&
 
 // api.cu: rows + entries per work unit when the caller names none, for `warps`
 // resident warps
-uint32_t choose_grain(uint64_t rows, uint64_t items, uint64_t warps, bool disperse);
+uint32_t choose_grain(uint64_t rows, uint64_t items, uint64_t warps, bool disperse, bool word);
 
 // coo.cu: Skipper over an edge list (src[i], dst[i]) in coordinate form
 struct CooParams {

@@ -435,7 +435,7 @@ mm_status mm_skipper_multi(mm_multi* m, uint64_t num_graphs, const mm_graph_desc
   const uint64_t state_bytes = word ? 4 * rows : rows * bits / 8;
   const bool fits = 2 * state_bytes <= (uint64_t)m->l2_bytes;
   const bool disperse = o->unit_order == MM_ORDER_DISPERSED || (o->unit_order == MM_ORDER_AUTO && fits);
-  const uint64_t grain = o->grain ? o->grain : choose_grain(rows, items, (uint64_t)m->num_sms * (fits ? 64 : 48), disperse);
+  const uint64_t grain = o->grain ? o->grain : choose_grain(rows, items, (uint64_t)m->num_sms * (fits ? 64 : 48), disperse, word);
   Layout L;
   if ((st = stage_tables(&m->sweep, num_graphs, h_descs, grain, (int)bits, s, &L)) != MM_OK) return st;
   MTRY(grow(&m->sweep.part, &m->sweep.part_cap, 2 * (L.units + 1), s));
