@@ -303,7 +303,7 @@ SweepParams make_params(mm_graph* g, const Resolved& r, uint32_t* d_mate) {
 // window, or a work split, block or occupancy of its own).
 bool chip_single(const mm_graph* g, const Resolved& r, const SweepParams& P) {
   return r.plain && !r.serial && !r.stats && !r.poison && !r.timing && !r.l2_persist && !P.sel && !P.tile &&
-         g->n + g->nnz <= kChipSingleItems;
+         g->n <= kChipSingleRows && g->n + g->nnz <= kChipSingleItems;
 }
 
 // The word a call that waits has its kernels report to; such calls on a handle
