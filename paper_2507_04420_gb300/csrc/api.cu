@@ -885,7 +885,7 @@ mm_status build_batch_graph(mm_graph* g, const Resolved& r, uint64_t num_graphs,
   b = BatchGraph{};
   CUDA_TRY(cudaGraphCreate(&b.graph, 0));
   const void *k_prepare = nullptr, *k_sweep = nullptr, *k_pairs = nullptr;
-  get_batched_kernels(r.bits, r.serial, P.sym != 0, P.lean != 0, &k_prepare, &k_sweep, &k_pairs);
+  get_batched_kernels(r.bits, r.serial, P.sym != 0, P.lean != 0, P.mesh != 0, &k_prepare, &k_sweep, &k_pairs);
 
   SweepParams p = P;
   uint64_t* gp = graph_pairs;
@@ -945,7 +945,7 @@ mm_status update_batch_graph(mm_graph* g, const Resolved& r, uint64_t num_graphs
                              const SweepParams& P, uint64_t* graph_pairs) {
   BatchGraph& b = g->bg;
   const void *k_prepare = nullptr, *k_sweep = nullptr, *k_pairs = nullptr;
-  get_batched_kernels(r.bits, r.serial, P.sym != 0, P.lean != 0, &k_prepare, &k_sweep, &k_pairs);
+  get_batched_kernels(r.bits, r.serial, P.sym != 0, P.lean != 0, P.mesh != 0, &k_prepare, &k_sweep, &k_pairs);
   SweepParams p = P;
   uint64_t* gp = graph_pairs;
   uint64_t ng = num_graphs;

@@ -252,13 +252,16 @@ cudaError_t launch_serial_batched(const SweepParams& P, int bits, cudaStream_t s
   return cudaGetLastError();
 }
 
-void get_batched_kernels(int bits, bool serial, bool sym, bool lean, const void** prepare,
+void get_batched_kernels(int bits, bool serial, bool sym, bool lean, bool mesh, const void** prepare,
                          const void** sweep, const void** pairs) {
 #define PK(S, B) (const void*)prepare_kernel<B>
 #define SB(S, B) (const void*)serial_batched_kernel<S>
-#define SW(S, B) (lean ? (const void*)sweep_kernel<S, false, false, false, false, true> : (const void*)sweep_kernel<S>)
-#define SY(S, B) (lean ? (const void*)sweep_kernel<S, false, true, false, false, true> \
-                       : (const void*)sweep_kernel<S, false, true>)
+#define SW(S, B) (mesh ? (const void*)sweep_kernel<S, false, false, false, false, true, true> \
+                  : lean ? (const void*)sweep_kernel<S, false, false, false, false, true> \
+                         : (const void*)sweep_kernel<S>)
+#define SY(S, B) (mesh ? (const void*)sweep_kernel<S, false, true, false, false, true, true> \
+                  : lean ? (const void*)sweep_kernel<S, false, true, false, false, true> \
+                         : (const void*)sweep_kernel<S, false, true>)
   *prepare = SKP_DISPATCH_STATE(bits, PK);
   *sweep = serial ? SKP_DISPATCH_STATE(bits, SB)
                   : sym ? SKP_DISPATCH_STATE(bits, SY) : SKP_DISPATCH_STATE(bits, SW);
