@@ -116,9 +116,11 @@ __device__ __forceinline__ uint32_t take_unit(unsigned long long* counter, uint6
 
 // Row end v of a CSR, kept inside the entries: graphs that were never checked
 // (MM_CHECK_CSR not given, local-id batches, multi-graph calls) may name others.
-__device__ __forceinline__ int64_t row_end(const int64_t* offsets, uint64_t v, uint64_t nnz) {
-  const int64_t e = __ldg(offsets + v);
+__device__ __forceinline__ int64_t clamp_end(int64_t e, uint64_t nnz) {
   return e < 0 ? 0 : e > (int64_t)nnz ? (int64_t)nnz : e;
+}
+__device__ __forceinline__ int64_t row_end(const int64_t* offsets, uint64_t v, uint64_t nnz) {
+  return clamp_end(__ldg(offsets + v), nnz);
 }
 
 // An error of the pass: into the device's word, which other warps look at, and,

@@ -395,15 +395,15 @@ __device__ __forceinline__ void serial_rows(const S& s, const SweepParams& P, ui
   int64_t next_at = -256;
   int64_t begin = 0, end = 0;           // row ends of the window after this one
   if (r0 + lane < r1) {
-    begin = row_end(P.offsets, r0 + lane, P.nnz);
-    end = row_end(P.offsets, r0 + lane + 1, P.nnz);
+    begin = __ldg(P.offsets + r0 + lane);
+    end = __ldg(P.offsets + r0 + lane + 1);
   }
   for (uint64_t wb = r0; wb < r1; wb += 32) {
     const bool in = wb + lane < r1;
-    const int64_t my_begin = begin, my_end = end;
+    const int64_t my_begin = clamp_end(begin, P.nnz), my_end = clamp_end(end, P.nnz);  // not on the load's heels
     if (wb + 32 + lane < r1) {
-      begin = row_end(P.offsets, wb + 32 + lane, P.nnz);
-      end = row_end(P.offsets, wb + 32 + lane + 1, P.nnz);
+      begin = __ldg(P.offsets + wb + 32 + lane);
+      end = __ldg(P.offsets + wb + 32 + lane + 1);
     }
     // the row states arrive beside the first chunk's: until then every row reads as open
     const uint32_t my_st = in ? s.raw((uint32_t)(wb + lane)) : 0u;
