@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(512, 3) coo_sweep_kernel(CooParams C) {
       for (int j = 0; j < 4; ++j) {
         live[j] = i0 + j < e_hi && x[j] != y[j];  // lines 6-7: loops are skipped
         if (live[j] && (x[j] >= n32 || y[j] >= n32)) {
-          report(P.err, P.host_err, kErrBadId);
+          report_bad_id(P.err, P.host_err);
           live[j] = false;
         }
         rx[j] = live[j] ? s.peek(x[j]) : 0u;
@@ -163,10 +163,12 @@ __global__ void coo_serial_kernel(CooParams C) {
   if (blockIdx.x != 0 || threadIdx.x != 0) return;
   const SweepParams& P = C.P;
   const S s(P);
+  bool told = false;
   for (uint64_t i = 0; i < C.m; ++i) {
     const uint32_t x = C.src[i], y = C.dst[i];
     if (x >= P.n || y >= P.n) {
-      report(P.err, P.host_err, kErrBadId);
+      if (!told) report(P.err, P.host_err, kErrBadId);
+      told = true;
       continue;
     }
     if (x == y) continue;

@@ -301,7 +301,7 @@ __device__ __forceinline__ void sweep_unit(const S& s, const SweepParams& P, int
       bad |= want[j] && y[j] >= n32;
       want[j] = want[j] && y[j] < n32;
     }
-    if (__any_sync(kFull, bad) && bad) report(P.err, P.host_err, kErrBadId);
+    if (__any_sync(kFull, bad) && bad) report_bad_id(P.err, P.host_err);
     uint32_t ry[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
     for (int j = 0; j < 4; ++j)
@@ -394,6 +394,7 @@ __device__ __forceinline__ void serial_rows(const S& s, const SweepParams& P, ui
   uint32_t next[4] = {0u, 0u, 0u, 0u};  // ids at next_at + 4 * lane
   int64_t next_at = -256;
   int64_t begin = 0, end = 0;           // row ends of the window after this one
+  bool told = false;                    // the lane has reported an id out of range
   if (r0 + lane < r1) {
     begin = __ldg(P.offsets + r0 + lane);
     end = __ldg(P.offsets + r0 + lane + 1);
@@ -469,7 +470,8 @@ __device__ __forceinline__ void serial_rows(const S& s, const SweepParams& P, ui
           if ((int)lane == first) {
             cand &= cand - 1u;
             if (yv >= n32) {
-              report(P.err, P.host_err, kErrBadId);
+              if (!told) report(P.err, P.host_err, kErrBadId);
+              told = true;
             } else if constexpr (S::kAlone) {  // both ends are free, or the entry had been dropped
               s.match_alone(xv, yv);
               got = 1u;
