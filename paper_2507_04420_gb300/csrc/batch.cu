@@ -279,6 +279,7 @@ __global__ void __launch_bounds__(256, kCheckBlocks) batch_check_kernel(BatchPar
   const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
   const uint64_t N = B.P.n, G = B.num_graphs;
   uint32_t matched = 0, pairs = 0;
+  init_counts(lane);
   for (uint64_t w0 = warp * 32 * kCheckRun; w0 < N; w0 += nwarps * 32 * kCheckRun) {
     uint64_t g = warp_last_at_or_below(B.vbase, G, w0, lane);
     for (uint64_t v0 = w0; v0 < w0 + 32 * kCheckRun && v0 < N; v0 += 32) {
@@ -291,7 +292,7 @@ __global__ void __launch_bounds__(256, kCheckBlocks) batch_check_kernel(BatchPar
       const Visit a = check_group<false>(V, in, v, load_vertex(V, in, v), (uint32_t)g, lane, queue);
       matched += __popc(__ballot_sync(kFull, a.bits & kVxMatched));
       pairs += __popc(__ballot_sync(kFull, a.bits & kVxPair));
-      add_faults(c, a, i, lane);
+      add_faults(a, i, lane);
     }
   }
   add_block(c, matched, pairs);
@@ -301,10 +302,12 @@ __global__ void __launch_bounds__(256, kCheckBlocks) batch_check_kernel(BatchPar
 __global__ void batch_check_long_kernel(BatchParams B, LongRows queue, unsigned long long* __restrict__ c,
                                         unsigned long long* __restrict__ host) {
   const unsigned long long rows = queue.size();
+  init_counts(threadIdx.x & 31u);
   for (unsigned long long i = 0; i < rows; ++i) {
     const uint64_t item = queue.items[i];
-    check_long_row(batch_check_view(B, item >> 32), (uint32_t)item, c, threadIdx.x & 31u);
+    check_long_row(batch_check_view(B, item >> 32), (uint32_t)item, threadIdx.x & 31u);
   }
+  add_block(c, 0, 0);
   publish_counters<true>(c, host);
 }
 

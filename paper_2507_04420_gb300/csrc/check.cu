@@ -71,13 +71,14 @@ __global__ void __launch_bounds__(256, kCheckBlocks) check_csr_kernel(CheckView 
   const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
   uint32_t matched = 0, pairs = 0;
+  init_counts(lane);
   for (uint64_t v0 = warp * 32; v0 < V.n; v0 += nwarps * 32) {
     const bool in = v0 + lane < V.n;
     const uint32_t v = (uint32_t)v0 + lane;
     const Visit a = check_group<true>(V, in, v, load_vertex(V, in, v), 0, lane, queue);
     matched += __popc(__ballot_sync(kFull, a.bits & kVxMatched));
     pairs += __popc(__ballot_sync(kFull, a.bits & kVxPair));
-    add_faults(c, a, v0 + lane, lane);
+    add_faults(a, v0 + lane, lane);
   }
   add_block(c, matched, pairs);
   publish_counters<false>(c, host);
@@ -87,8 +88,9 @@ __global__ void __launch_bounds__(256, kCheckBlocks) check_csr_kernel(CheckView 
 __global__ void check_csr_long_kernel(CheckView V, LongRows queue, unsigned long long* __restrict__ c,
                                       unsigned long long* __restrict__ host) {
   const unsigned long long rows = queue.size();
-  for (unsigned long long i = 0; i < rows; ++i)
-    check_long_row(V, (uint32_t)queue.items[i], c, threadIdx.x & 31u);
+  init_counts(threadIdx.x & 31u);
+  for (unsigned long long i = 0; i < rows; ++i) check_long_row(V, (uint32_t)queue.items[i], threadIdx.x & 31u);
+  add_block(c, 0, 0);
   publish_counters<true>(c, host);
 }
 
@@ -135,6 +137,7 @@ __global__ void validate_coo_vertex_kernel(uint64_t n, const uint32_t* __restric
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   const unsigned lane = threadIdx.x & 31u;
   uint32_t matched = 0, pairs = 0;
+  init_counts(lane);
   for (uint64_t v0 = (uint64_t)blockIdx.x * blockDim.x; v0 < n; v0 += stride) {
     const uint64_t v = v0 + threadIdx.x;
     const uint32_t m = v < n ? mate[v] : kNone;
@@ -149,7 +152,7 @@ __global__ void validate_coo_vertex_kernel(uint64_t n, const uint32_t* __restric
     }
     matched += __popc(__ballot_sync(kFull, a.bits & kVxMatched));
     pairs += __popc(__ballot_sync(kFull, a.bits & kVxPair));
-    add_faults(c, a, v, lane);
+    add_faults(a, v, lane);
   }
   add_block(c, matched, pairs);
   publish_counters<true>(c, host);

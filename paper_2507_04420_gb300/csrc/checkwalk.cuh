@@ -276,10 +276,22 @@ __device__ __forceinline__ void add_nonzero(unsigned long long* c, unsigned long
   if (v) atomicAdd(c, v);
 }
 
-// The faults of one visit, each lane's vertex reported as index `at`, into
-// counters that all lanes share (every lane takes part).
-__device__ __forceinline__ void add_faults(unsigned long long* c, const Visit& a, unsigned long long at,
-                                           unsigned lane) {
+// What a warp has counted so far, in shared memory (blocks of 256 threads):
+// added to the verdict's counters when it is done, not group by group -- a wrong
+// matching has faults in every group, and 2.5 M pairs of atomics on two words
+// took most of the check of an empty matching of a 9000 x 9000 grid.
+__device__ __forceinline__ unsigned long long* warp_counts() {
+  __shared__ unsigned long long counts[8][kCkCount];
+  return counts[threadIdx.x >> 5];
+}
+__device__ __forceinline__ void init_counts(unsigned lane) {
+  if (lane < kCkCount) warp_counts()[lane] = 0ull;
+  __syncwarp();
+}
+
+// The faults of one visit, each lane's vertex reported as index `at`, into the
+// warp's counts (every lane takes part).
+__device__ __forceinline__ void add_faults(const Visit& a, unsigned long long at, unsigned lane) {
   if (!__any_sync(kFull, (a.bits & kVxBad) != 0u || a.uncovered != 0u)) return;
   const uint32_t range = __popc(__ballot_sync(kFull, a.bits & kVxRange));
   const uint32_t asym = __popc(__ballot_sync(kFull, a.bits & kVxAsym));
@@ -288,41 +300,54 @@ __device__ __forceinline__ void add_faults(unsigned long long* c, const Visit& a
   const uint32_t uncovered = __reduce_add_sync(kFull, a.uncovered);
   const unsigned long long bad = warp_min64(a.bits & kVxBad ? at : ~0ull), unc = warp_min64(a.first_unc);
   if (lane == 0) {
-    add_nonzero(c + kCkRange, range);
-    add_nonzero(c + kCkAsym, asym);
-    add_nonzero(c + kCkNonedge, nonedge);
-    add_nonzero(c + kCkUncovered, uncovered);
-    if (~bad) atomicMax(c + kCkFirstBad, ~bad);
-    if (~unc) atomicMax(c + kCkFirstUncovered, ~unc);
+    unsigned long long* const c = warp_counts();
+    c[kCkRange] += range;
+    c[kCkAsym] += asym;
+    c[kCkNonedge] += nonedge;
+    c[kCkUncovered] += uncovered;
+    if (~bad > c[kCkFirstBad]) c[kCkFirstBad] = ~bad;
+    if (~unc > c[kCkFirstUncovered]) c[kCkFirstUncovered] = ~unc;
   }
 }
 
+// The warp's counts into counters `c`, and the warp's left at zero.
+__device__ __forceinline__ void flush_counts(unsigned long long* c, unsigned lane) {
+  __syncwarp();
+  if (lane < kCkCount) {
+    const unsigned long long v = warp_counts()[lane];
+    if (v) lane < kCkFirstBad ? atomicAdd(c + lane, v) : atomicMax(c + lane, v);
+    warp_counts()[lane] = 0ull;
+  }
+  __syncwarp();
+}
+
 // One queued row, spread over the whole grid.
-__device__ __forceinline__ void check_long_row(const CheckView& V, uint32_t x, unsigned long long* c,
-                                               unsigned lane) {
+__device__ __forceinline__ void check_long_row(const CheckView& V, uint32_t x, unsigned lane) {
   const int64_t s = V.end(x), e = V.end((uint64_t)x + 1);
   const int64_t step = 4 * (int64_t)gridDim.x * blockDim.x;
   Visit a;  // an entry in 4 * step: 32 bits hold a lane's share
   for (int64_t q = (s & ~(int64_t)3) + 4 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x); q < e; q += step)
     quad_scan(check_quad(V.nbrs, V.nnz, q, e), q, s, e, x, V.mate, V.n, a);
-  add_faults(c, a, 0, lane);
+  add_faults(a, 0, lane);
 }
 
-// A block's matched vertices and pairs (each warp's on all its lanes), added
-// once a block: added a warp at a time, the counts of 16.8 M vertices took
-// most of a 0.69 ms pass.
+// A block's counts, with its matched vertices and pairs (each warp's on all its
+// lanes), added once a block: added a warp at a time, the counts of 16.8 M
+// vertices took most of a 0.69 ms pass.
 __device__ __forceinline__ void add_block(unsigned long long* c, uint32_t matched, uint32_t pairs) {
-  __shared__ uint32_t sum[2][32];
-  const unsigned warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   if ((threadIdx.x & 31u) == 0) {
-    sum[0][warp] = matched;
-    sum[1][warp] = pairs;
+    warp_counts()[kCkMatched] += matched;
+    warp_counts()[kCkPairs] += pairs;
   }
   __syncthreads();
-  if (threadIdx.x < 2) {
+  if (threadIdx.x < kCkCount) {
+    const unsigned long long* const at = warp_counts() + threadIdx.x;  // the first warp's; the others' lie behind
     unsigned long long t = 0;
-    for (unsigned w = 0; w < nw; ++w) t += sum[threadIdx.x][w];
-    add_nonzero(c + (threadIdx.x ? kCkPairs : kCkMatched), t);
+    for (unsigned w = 0; w < blockDim.x >> 5; ++w) {
+      const unsigned long long v = at[w * kCkCount];
+      t = threadIdx.x < kCkFirstBad ? t + v : v > t ? v : t;
+    }
+    if (t) threadIdx.x < kCkFirstBad ? atomicAdd(c + threadIdx.x, t) : atomicMax(c + threadIdx.x, t);
   }
 }
 

@@ -153,8 +153,8 @@ __device__ __forceinline__ void group_add(unsigned long long* c, unsigned peers,
 
 // The exact checker (checkwalk.cuh) over every vertex of every graph, one set
 // of counters a graph.  A warp takes runs of kCheckRun * 32 consecutive
-// vertices of the whole batch: one search finds a run's graph, and its sums go
-// to the graph's counters when the run leaves it, not vertex by vertex.
+// vertices of the whole batch: one search finds a run's graph, and its counts go
+// to the graph's counters when the warp leaves it, not vertex by vertex.
 constexpr uint64_t kCheckRun = 4;  // 8: 195 us for 171 graphs of up to 1e6 edges; 4: 165
 
 __device__ __forceinline__ CheckView multi_check_view(const MultiParams& M, uint64_t g) {
@@ -167,17 +167,10 @@ __global__ void __launch_bounds__(256, kCheckBlocks) multi_check_kernel(MultiPar
   const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
   const uint64_t G = M.num_graphs, N = M.vbase[G];
+  init_counts(lane);
+  uint64_t cur = 0;  // the graph of the warp's counts
   for (uint64_t w0 = warp * 32 * kCheckRun; w0 < N; w0 += nwarps * 32 * kCheckRun) {
     uint64_t g = warp_last_at_or_below(M.vbase, G, w0, lane);
-    uint64_t cur = g;  // the graph of the sums
-    uint32_t matched = 0, pairs = 0;
-    auto flush = [&]() {
-      if (lane == 0) {
-        add_nonzero(M.counters + cur * kCkCount + kCkMatched, matched);
-        add_nonzero(M.counters + cur * kCkCount + kCkPairs, pairs);
-      }
-      matched = pairs = 0;
-    };
     for (uint64_t v0 = w0; v0 < w0 + 32 * kCheckRun && v0 < N; v0 += 32) {
       const uint64_t i = v0 + lane;
       const bool in = i < N;
@@ -188,11 +181,14 @@ __global__ void __launch_bounds__(256, kCheckBlocks) multi_check_kernel(MultiPar
       const uint64_t g0 = __shfl_sync(kFull, g, 0);
       const unsigned active = __ballot_sync(kFull, in);
       if (__all_sync(kFull, !in || g == g0)) {
-        if (g0 != cur) flush();
+        if (g0 != cur) flush_counts(M.counters + cur * kCkCount, lane);
         cur = g0;
-        matched += __popc(__ballot_sync(kFull, a.bits & kVxMatched));
-        pairs += __popc(__ballot_sync(kFull, a.bits & kVxPair));
-        add_faults(M.counters + g0 * kCkCount, a, v, lane);
+        const unsigned matched = __ballot_sync(kFull, a.bits & kVxMatched), pairs = __ballot_sync(kFull, a.bits & kVxPair);
+        if (lane == 0) {
+          warp_counts()[kCkMatched] += __popc(matched);
+          warp_counts()[kCkPairs] += __popc(pairs);
+        }
+        add_faults(a, v, lane);
       } else if (in) {  // the group spans graphs: each lane counts for its own
         unsigned long long* c = M.counters + g * kCkCount;
         const unsigned peers = __match_any_sync(active, g);
@@ -207,16 +203,17 @@ __global__ void __launch_bounds__(256, kCheckBlocks) multi_check_kernel(MultiPar
       }
       g = __shfl_sync(kFull, g, 0);
     }
-    flush();
   }
+  flush_counts(M.counters + cur * kCkCount, lane);
 }
 
 __global__ void multi_check_long_kernel(MultiParams M, LongRows queue) {
   const unsigned long long rows = queue.size();
+  init_counts(threadIdx.x & 31u);
   for (unsigned long long i = 0; i < rows; ++i) {
     const uint64_t item = queue.items[i];
-    check_long_row(multi_check_view(M, item >> 32), (uint32_t)item, M.counters + (item >> 32) * kCkCount,
-                   threadIdx.x & 31u);
+    check_long_row(multi_check_view(M, item >> 32), (uint32_t)item, threadIdx.x & 31u);
+    flush_counts(M.counters + (item >> 32) * kCkCount, threadIdx.x & 31u);
   }
 }
 
