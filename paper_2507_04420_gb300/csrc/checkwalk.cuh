@@ -42,13 +42,15 @@ namespace {
 // 8 / 16 / 32 quads: the 4096-graph batch's check 339 / 324 / 320 us, R-MAT 22's 170 / 174 / 185
 constexpr int64_t kLaneQuads = 16;
 
-// a graph as the checker reads it (nbrs 16-byte aligned, nnz entries in all)
+// a graph as the checker reads it (nbrs 16-byte aligned, nnz entries in all).  Row
+// ends that were never checked may lie anywhere: a position outside the entries
+// holds no id (check_quad), and rows longer than a lane takes are clamped before
+// they are walked.  Clamping every row as it is loaded cost 12 to 17% on lattices.
 struct CheckView {
   const int64_t* offsets;
   const uint32_t* nbrs;
   const uint32_t* mate;
   uint64_t n, nnz;
-  __device__ __forceinline__ int64_t end(uint64_t v) const { return row_end(offsets, v, nnz); }
 };
 
 // what one visit found: the vertex's bits, and the uncovered entries this lane met
@@ -108,14 +110,16 @@ __device__ __forceinline__ unsigned long long warp_min64(unsigned long long v) {
   return v;
 }
 
-// the ids at [q, q + 4), q a multiple of 4, as far as they exist before `e` or lie in a whole quad
+// the ids at [q, q + 4), q a multiple of 4 below `e`; kNone, which is no vertex, where no entry is
 __device__ __forceinline__ uint4 check_quad(const uint32_t* nbrs, uint64_t nnz, int64_t q, int64_t e) {
-  uint4 y = make_uint4(0u, 0u, 0u, 0u);
+  uint4 y = make_uint4(kNone, kNone, kNone, kNone);
   if (q >= e) return y;
-  if (q + 4 <= (int64_t)nnz) return __ldg(reinterpret_cast<const uint4*>(nbrs + q));
-  y.x = __ldg(nbrs + q);
-  if (q + 1 < e) y.y = __ldg(nbrs + q + 1);
-  if (q + 2 < e) y.z = __ldg(nbrs + q + 2);
+  const uint64_t whole = nnz & ~3ull;  // entries in whole quads
+  if ((uint64_t)q < whole) return __ldg(reinterpret_cast<const uint4*>(nbrs + q));
+  if ((uint64_t)q != whole) return y;
+  if (whole < nnz) y.x = __ldg(nbrs + q);
+  if (whole + 1 < nnz) y.y = __ldg(nbrs + q + 1);
+  if (whole + 2 < nnz) y.z = __ldg(nbrs + q + 2);
   return y;
 }
 
@@ -169,8 +173,8 @@ __device__ __forceinline__ VertexRow load_vertex(const CheckView& V, bool in, ui
   VertexRow r;
   if (in) {
     r.m = __ldg(V.mate + v);
-    r.s = V.end(v);
-    r.e = V.end((uint64_t)v + 1);
+    r.s = __ldg(V.offsets + v);
+    r.e = __ldg(V.offsets + v + 1);
   }
   return r;
 }
@@ -192,7 +196,7 @@ __device__ __forceinline__ Visit check_group(const CheckView& V, bool in, uint32
       a.bits = kVxMatched | (sym ? kVxBothEnds | (v < m ? kVxPair : 0u) : kVxAsym);
       find = !sym || v < m;
       if (find) {
-        const int64_t s2 = V.end(m), e2 = V.end((uint64_t)m + 1);
+        const int64_t s2 = __ldg(V.offsets + m), e2 = __ldg(V.offsets + m + 1);
         if (e2 - s2 < e - s) {             // the shorter row first
           s = s2;
           e = e2;
@@ -203,7 +207,7 @@ __device__ __forceinline__ Visit check_group(const CheckView& V, bool in, uint32
   }
   bool todo = find || (in && m == kNone && s < e);
   for (;;) {  // short rows: one a lane
-    const bool mine = todo && ((e + 3) >> 2) - (s >> 2) <= kLaneQuads;
+    const bool mine = todo && ((e - 1) >> 2) - (s >> 2) < kLaneQuads;
     if (!__any_sync(kFull, mine)) break;
     if (!mine) continue;
     const int64_t q = s & ~(int64_t)3;
@@ -221,8 +225,8 @@ __device__ __forceinline__ Visit check_group(const CheckView& V, bool in, uint32
     if (s < e) continue;
     if (find && again) {
       again = false;
-      s = V.end(t);
-      e = V.end((uint64_t)t + 1);
+      s = __ldg(V.offsets + t);
+      e = __ldg(V.offsets + t + 1);
       t ^= other;
     } else {
       todo = false;
@@ -233,9 +237,9 @@ __device__ __forceinline__ Visit check_group(const CheckView& V, bool in, uint32
   while (left) {  // longer rows: the warp reads one at a time
     const int j = __ffs(left) - 1;
     left &= left - 1;
-    const int64_t sj = __shfl_sync(kFull, s, j), ej = __shfl_sync(kFull, e, j);
     const uint32_t* nbrs = kOne ? V.nbrs : shfl_ptr(V.nbrs, j);
     const uint64_t nnz = kOne ? V.nnz : __shfl_sync(kFull, V.nnz, j);
+    const int64_t sj = clamp_end(__shfl_sync(kFull, s, j), nnz), ej = clamp_end(__shfl_sync(kFull, e, j), nnz);
     if (__shfl_sync(kFull, find ? 1 : 0, j)) {
       const uint32_t tj = __shfl_sync(kFull, t, j), oj = __shfl_sync(kFull, other, j);
       bool hit = warp_row_has(nbrs, nnz, sj, ej, tj, lane);
@@ -323,7 +327,7 @@ __device__ __forceinline__ void flush_counts(unsigned long long* c, unsigned lan
 
 // One queued row, spread over the whole grid.
 __device__ __forceinline__ void check_long_row(const CheckView& V, uint32_t x, unsigned lane) {
-  const int64_t s = V.end(x), e = V.end((uint64_t)x + 1);
+  const int64_t s = row_end(V.offsets, x, V.nnz), e = row_end(V.offsets, (uint64_t)x + 1, V.nnz);
   const int64_t step = 4 * (int64_t)gridDim.x * blockDim.x;
   Visit a;  // an entry in 4 * step: 32 bits hold a lane's share
   for (int64_t q = (s & ~(int64_t)3) + 4 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x); q < e; q += step)
