@@ -86,7 +86,7 @@ struct mm_graph {
   int last_bits = 0;                   // layout and state array of the last mm_skipper call
   const uint32_t* last_state = nullptr;
   unsigned char* found = nullptr;      // checker scratch, allocated on first mm_validate
-  uint64_t* long_rows = nullptr;
+  ulonglong2* long_rows = nullptr;
   uint64_t* tiles = nullptr;           // compaction words (compact_words)
   uint32_t* h_err = nullptr;           // pinned: [0] status of the last call, [1] of a call that waits
   unsigned long long* h_counters = nullptr;  // pinned, 16 words
@@ -1247,8 +1247,8 @@ mm_status mm_skipper_batched(mm_graph* g, uint64_t num_graphs, const int64_t* d_
 }
 
 static mm_status ensure_long_rows(mm_graph* g) {
-  const uint64_t cap = long_row_cap(g->nnz);
-  if (cap && !g->long_rows) CUDA_TRY(cudaMalloc(&g->long_rows, cap * sizeof(uint64_t)));
+  const uint64_t cap = long_row_cap(g->nnz, !g->local_ids);
+  if (cap && !g->long_rows) CUDA_TRY(cudaMalloc(&g->long_rows, cap * sizeof(ulonglong2)));
   return MM_OK;
 }
 

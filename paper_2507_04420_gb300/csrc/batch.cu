@@ -301,11 +301,11 @@ __global__ void __launch_bounds__(256, kCheckBlocks) batch_check_kernel(BatchPar
 
 __global__ void batch_check_long_kernel(BatchParams B, LongRows queue, unsigned long long* __restrict__ c,
                                         unsigned long long* __restrict__ host) {
-  const unsigned long long rows = queue.size();
+  const unsigned long long pieces = queue.size();
   init_counts(threadIdx.x & 31u);
-  for (unsigned long long i = 0; i < rows; ++i) {
-    const uint64_t item = queue.items[i];
-    check_long_row(batch_check_view(B, item >> 32), (uint32_t)item, threadIdx.x & 31u);
+  for (unsigned long long i = blockIdx.x; i < pieces; i += gridDim.x) {
+    const ulonglong2 item = queue.items[i];
+    check_piece(batch_check_view(B, item.x >> 32), (uint32_t)item.x, (int64_t)item.y, threadIdx.x & 31u);
   }
   add_block(c, 0, 0);
   publish_counters<true>(c, host);
@@ -349,14 +349,14 @@ int batch_sweep_blocks_per_sm(int bits, bool local, bool sym, bool lean, int blo
 }
 
 cudaError_t launch_validate_batch(const BatchParams& B, const CheckScratch& cs, int sms, cudaStream_t s) {
-  const LongRows queue{cs.counters + kCkLong, cs.long_rows, long_row_cap(B.P.nnz)};
+  const LongRows queue{cs.counters + kCkLong, cs.long_rows, long_row_cap(B.P.nnz, false)};
   batch_check_kernel<<<check_grid(B.P.n, sms), 256, 0, s>>>(B, queue, cs.counters, cs.host);
   return cudaGetLastError();
 }
 
 cudaError_t launch_validate_batch_long(const BatchParams& B, const CheckScratch& cs, int sms, cudaStream_t s) {
   batch_check_long_kernel<<<sms * 4, 256, 0, s>>>(
-      B, LongRows{cs.counters + kCkLong, cs.long_rows, long_row_cap(B.P.nnz)}, cs.counters, cs.host);
+      B, LongRows{cs.counters + kCkLong, cs.long_rows, long_row_cap(B.P.nnz, false)}, cs.counters, cs.host);
   return cudaGetLastError();
 }
 

@@ -84,12 +84,15 @@ __global__ void __launch_bounds__(256, kCheckBlocks) check_csr_kernel(CheckView 
   publish_counters<false>(c, host);
 }
 
-// the queued rows of unmatched vertices, each spread over the grid
+// the queued pieces of unmatched vertices' rows, one a block
 __global__ void check_csr_long_kernel(CheckView V, LongRows queue, unsigned long long* __restrict__ c,
                                       unsigned long long* __restrict__ host) {
-  const unsigned long long rows = queue.size();
+  const unsigned long long pieces = queue.size();
   init_counts(threadIdx.x & 31u);
-  for (unsigned long long i = 0; i < rows; ++i) check_long_row(V, (uint32_t)queue.items[i], threadIdx.x & 31u);
+  for (unsigned long long i = blockIdx.x; i < pieces; i += gridDim.x) {
+    const ulonglong2 item = queue.items[i];
+    check_piece(V, (uint32_t)item.x, (int64_t)item.y, threadIdx.x & 31u);
+  }
   add_block(c, 0, 0);
   publish_counters<true>(c, host);
 }
@@ -324,8 +327,12 @@ __global__ void __launch_bounds__(kCompactThreads, 2) compact_kernel(uint64_t n,
 
 }  // namespace
 
-// rows of a CSR with nnz entries that can be longer than kLongRow
-uint64_t long_row_cap(uint64_t nnz) { return nnz / (uint64_t)kLongRow; }
+// pieces that the long rows of a CSR with nnz entries can have: those that a row fills,
+// and one more a row
+uint64_t long_row_cap(uint64_t nnz, bool one) {
+  const uint64_t row = (uint64_t)long_row(one);
+  return nnz > row ? nnz / (uint64_t)kPiece + nnz / row : 0;
+}
 
 // blocks of 256 threads for n vertices: no more than their groups of 32 fill, or than are resident
 int check_grid(uint64_t n, int sms) {
@@ -350,7 +357,7 @@ cudaError_t launch_validate(uint64_t n, uint64_t nnz, const int64_t* offsets, co
     validate_pairs_kernel<<<grid, 256, 0, s>>>(n, mate, pairs, count, cs.seen_bits, cs.counters);
   }
   const CheckView V{offsets, nbrs, mate, n, nnz};
-  const LongRows queue{cs.counters + kCkLong, cs.long_rows, long_row_cap(nnz)};
+  const LongRows queue{cs.counters + kCkLong, cs.long_rows, long_row_cap(nnz, true)};
   check_csr_kernel<<<check_grid(n, sms), 256, 0, s>>>(V, queue, cs.counters, cs.host);
   return cudaGetLastError();
 }
@@ -360,7 +367,7 @@ bool validate_needs_long(const CheckScratch& cs) { return cs.host[kCkLong] != 0;
 cudaError_t launch_validate_long(uint64_t n, uint64_t nnz, const int64_t* offsets, const uint32_t* nbrs,
                                  const uint32_t* mate, const CheckScratch& cs, int sms, cudaStream_t s) {
   check_csr_long_kernel<<<sms * 4, 256, 0, s>>>(CheckView{offsets, nbrs, mate, n, nnz},
-                                                LongRows{cs.counters + kCkLong, cs.long_rows, long_row_cap(nnz)},
+                                                LongRows{cs.counters + kCkLong, cs.long_rows, long_row_cap(nnz, true)},
                                                 cs.counters, cs.host);
   return cudaGetLastError();
 }

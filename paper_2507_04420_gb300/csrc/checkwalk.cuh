@@ -16,9 +16,8 @@
 // ids, then their mates -- and most rows it reads are a few entries long, so a
 // lane reads its own row, 8 entries a step, which keeps 32 rows in flight a
 // warp; a row of more than kLaneQuads quads is read by the whole warp, 256
-// entries a step.  A row of an unmatched vertex longer than kLongRow entries
-// (hubs, in matchings that are not maximal) is left to a second kernel that
-// spreads it over the GPU.
+// entries a step.  A row of an unmatched vertex longer than long_row entries
+// is cut into pieces, which a second kernel hands to the GPU's blocks.
 #pragma once
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -34,7 +33,11 @@ enum CheckSlot : int { kCkMatched = 0, kCkPairs, kCkRange, kCkAsym, kCkNonedge, 
                        kCkFirstBad, kCkFirstUncovered, kCkCount,
                        // control words behind them: long rows queued, blocks done
                        kCkLong = kCkCount, kCkDone, kCkWords };
-constexpr int64_t kLongRow = 16384;  // entries; see above
+constexpr int64_t kPiece = 8192;     // entries of a piece of a long row, at most (4096, 2048: 18 and 33% slower)
+// Entries from which a row is long: over one graph a warp keeps up with up to a
+// piece; over many, where it also fetches each row's graph from another lane, with
+// less (40,000 rows of 3000 entries: 1560 us by warps, 690 in pieces).
+__host__ __device__ constexpr int64_t long_row(bool one) { return one ? kPiece : 2048; }
 constexpr int kCheckBlocks = 5;      // resident blocks of 256 threads an SM (4 and 6 are 5 to 10% slower)
 
 namespace {
@@ -62,20 +65,34 @@ struct Visit {
   unsigned long long first_unc = ~0ull;
 };
 
-// rows of unmatched vertices left to the second kernel: graph << 32 | vertex.
-// cap counts the rows that can be so long when none overlap; row ends that were
-// never checked may overlap, and what does not fit is read at once.
+// Pieces of long rows of unmatched vertices, left to the second kernel: graph <<
+// 32 | vertex, and the number of the piece in its row.  A row spread over the
+// whole grid a row at a time kept only the blocks its length reached at work, and
+// all of them walking the queue: 39,000 rows of 17,000 to 22,000 entries 44.5 ms,
+// in pieces 1.25.  cap counts the pieces of rows that do not overlap; row ends
+// that were never checked may, and what does not fit is read at once.
 struct LongRows {
   unsigned long long* count;
-  uint64_t* items;
+  ulonglong2* items;
   uint64_t cap;
-  __device__ __forceinline__ bool push(uint64_t item) const {
-    const unsigned long long at = atomicAdd(count, 1ull);
-    if (at < cap) items[at] = item;
-    return at < cap;
+  // the whole warp queues the k pieces of a row; returns how many fitted
+  __device__ __forceinline__ int64_t push(uint64_t row, int64_t k, unsigned lane) const {
+    unsigned long long at = 0;
+    if (lane == 0) at = atomicAdd(count, (unsigned long long)k);
+    at = __shfl_sync(kFull, at, 0);
+    const int64_t fit = at >= cap ? 0 : (uint64_t)k < cap - at ? k : (int64_t)(cap - at);
+    for (int64_t i = lane; i < fit; i += 32) items[at + i] = make_ulonglong2(row, (unsigned long long)i);
+    return fit;
   }
   __device__ __forceinline__ unsigned long long size() const { return *count < cap ? *count : cap; }
 };
+
+// a row of `len` entries in pieces of at most kPiece, all but the last of one length
+__device__ __forceinline__ int64_t long_pieces(int64_t len) { return (len + kPiece - 1) / kPiece; }
+__device__ __forceinline__ int64_t piece_length(int64_t len) {
+  const int64_t k = long_pieces(len);
+  return (len + k - 1) / k;
+}
 
 // last g < G with base[g] <= x (base ascending, base[0] = 0 <= x < base[G]), found by the whole warp;
 // some g < G whatever base holds
@@ -239,7 +256,8 @@ __device__ __forceinline__ Visit check_group(const CheckView& V, bool in, uint32
     left &= left - 1;
     const uint32_t* nbrs = kOne ? V.nbrs : shfl_ptr(V.nbrs, j);
     const uint64_t nnz = kOne ? V.nnz : __shfl_sync(kFull, V.nnz, j);
-    const int64_t sj = clamp_end(__shfl_sync(kFull, s, j), nnz), ej = clamp_end(__shfl_sync(kFull, e, j), nnz);
+    int64_t sj = clamp_end(__shfl_sync(kFull, s, j), nnz);
+    const int64_t ej = clamp_end(__shfl_sync(kFull, e, j), nnz);
     if (__shfl_sync(kFull, find ? 1 : 0, j)) {
       const uint32_t tj = __shfl_sync(kFull, t, j), oj = __shfl_sync(kFull, other, j);
       bool hit = warp_row_has(nbrs, nnz, sj, ej, tj, lane);
@@ -248,9 +266,14 @@ __device__ __forceinline__ Visit check_group(const CheckView& V, bool in, uint32
         hit = warp_row_has(nbrs, nnz, row_end(offsets, tj, nnz), row_end(offsets, (uint64_t)tj + 1, nnz), tj ^ oj, lane);
       }
       if (!hit && (int)lane == j) a.bits |= kVxNonedge;
-    } else if (ej - sj <= kLongRow ||
-               !__shfl_sync(kFull, (int)lane == j && queue.push((uint64_t)graph << 32 | v) ? 1 : 0, j)) {
+    } else {
       const uint32_t xj = __shfl_sync(kFull, v, j);
+      if (ej - sj > long_row(kOne)) {
+        const int64_t k = long_pieces(ej - sj);
+        const int64_t fit = queue.push((uint64_t)__shfl_sync(kFull, graph, j) << 32 | xj, k, lane);
+        if (fit == k) continue;
+        sj += fit * piece_length(ej - sj);
+      }
       const uint32_t* mate = kOne ? V.mate : shfl_ptr(V.mate, j);
       const uint64_t n = kOne ? V.n : __shfl_sync(kFull, V.n, j);
       Visit part;
@@ -325,13 +348,17 @@ __device__ __forceinline__ void flush_counts(unsigned long long* c, unsigned lan
   __syncwarp();
 }
 
-// One queued row, spread over the whole grid.
-__device__ __forceinline__ void check_long_row(const CheckView& V, uint32_t x, unsigned lane) {
-  const int64_t s = row_end(V.offsets, x, V.nnz), e = row_end(V.offsets, (uint64_t)x + 1, V.nnz);
-  const int64_t step = 4 * (int64_t)gridDim.x * blockDim.x;
-  Visit a;  // an entry in 4 * step: 32 bits hold a lane's share
-  for (int64_t q = (s & ~(int64_t)3) + 4 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x); q < e; q += step)
-    quad_scan(check_quad(V.nbrs, V.nnz, q, e), q, s, e, x, V.mate, V.n, a);
+// One queued piece of row x, read by a block.
+__device__ __forceinline__ void check_piece(const CheckView& V, uint32_t x, int64_t piece, unsigned lane) {
+  const int64_t s0 = row_end(V.offsets, x, V.nnz), e0 = row_end(V.offsets, (uint64_t)x + 1, V.nnz);
+  const int64_t step = piece_length(e0 - s0), s = s0 + piece * step, e = s + step < e0 ? s + step : e0;
+  Visit a;
+  for (int64_t q = (s & ~(int64_t)3) + 4 * (int64_t)threadIdx.x; q < e; q += 8 * (int64_t)blockDim.x) {
+    const int64_t p = q + 4 * (int64_t)blockDim.x;
+    const uint4 y0 = check_quad(V.nbrs, V.nnz, q, e), y1 = check_quad(V.nbrs, V.nnz, p, e);
+    quad_scan(y0, q, s, e, x, V.mate, V.n, a);
+    quad_scan(y1, p, s, e, x, V.mate, V.n, a);
+  }
   add_faults(a, 0, lane);
 }
 

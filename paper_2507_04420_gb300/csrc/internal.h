@@ -86,9 +86,9 @@ struct CheckScratch {
   unsigned long long* host;      // page-locked: the finished counters, in mm_verdict's order after the flags
   uint32_t* seen_bits;           // ceil(n/32) words
   unsigned char* found;          // edge-list checker: n bytes (+3), partner edge met in the list
-  uint64_t* long_rows;           // CSR checker: long_row_cap(nnz) entries, null when that is 0
+  ulonglong2* long_rows;         // CSR checker: long_row_cap pieces of rows, null when that is 0
 };
-uint64_t long_row_cap(uint64_t nnz);
+uint64_t long_row_cap(uint64_t nnz, bool one);  // one: a CSR checked as one graph
 int check_grid(uint64_t n, int sms);
 cudaError_t launch_csr_check(uint64_t n, uint64_t nnz, const int64_t* offsets,
                              const uint32_t* nbrs, unsigned long long* bad, int grid,

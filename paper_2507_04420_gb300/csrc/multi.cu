@@ -208,13 +208,17 @@ __global__ void __launch_bounds__(256, kCheckBlocks) multi_check_kernel(MultiPar
 }
 
 __global__ void multi_check_long_kernel(MultiParams M, LongRows queue) {
-  const unsigned long long rows = queue.size();
+  const unsigned long long pieces = queue.size();
   init_counts(threadIdx.x & 31u);
-  for (unsigned long long i = 0; i < rows; ++i) {
-    const uint64_t item = queue.items[i];
-    check_long_row(multi_check_view(M, item >> 32), (uint32_t)item, threadIdx.x & 31u);
-    flush_counts(M.counters + (item >> 32) * kCkCount, threadIdx.x & 31u);
+  uint64_t cur = 0;  // the graph of the counts
+  for (unsigned long long i = blockIdx.x; i < pieces; i += gridDim.x) {
+    const ulonglong2 item = queue.items[i];
+    const uint64_t g = item.x >> 32;
+    if (g != cur) flush_counts(M.counters + cur * kCkCount, threadIdx.x & 31u);
+    cur = g;
+    check_piece(multi_check_view(M, g), (uint32_t)item.x, (int64_t)item.y, threadIdx.x & 31u);
   }
+  flush_counts(M.counters + cur * kCkCount, threadIdx.x & 31u);
 }
 
 // Grow a device buffer to at least `want` elements, ordered on the call's
@@ -299,7 +303,7 @@ struct Layout {
   uint64_t bytes = 0;
   uint64_t off_ubase = 0, off_vbase = 0, off_sbase = 0;
   uint64_t total_vertices = 0, total_words = 0;
-  uint64_t long_rows = 0;              // rows that can be longer than kLongRow
+  uint64_t long_rows = 0;              // pieces that long rows can have
 };
 
 mm_status stage_tables(TableSet* m, uint64_t G, const mm_graph_desc* h, uint64_t grain, int bits,
@@ -330,7 +334,7 @@ mm_status stage_tables(TableSet* m, uint64_t G, const mm_graph_desc* h, uint64_t
   for (uint64_t g = 0; g < G; ++g) {
     ub[g + 1] = ub[g] + (h[g].n + h[g].nnz + grain - 1) / grain;
     vb[g + 1] = vb[g] + h[g].n;
-    L->long_rows += long_row_cap(h[g].nnz);
+    L->long_rows += long_row_cap(h[g].nnz, false);
     sb[g + 1] = sb[g] + (bits == 32 ? 0 : packed_words(h[g].n, bits) + 1);
   }
   L->units = ub[G];
@@ -499,10 +503,10 @@ mm_status mm_validate_multi_async(mm_multi* m, uint64_t num_graphs, const mm_gra
   if (st != MM_OK) return st;
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   Layout L;
-  if ((st = stage_tables(&m->check, num_graphs, h_descs, (uint64_t)kLongRow, 32, s, &L)) != MM_OK) return st;
+  if ((st = stage_tables(&m->check, num_graphs, h_descs, (uint64_t)kPiece, 32, s, &L)) != MM_OK) return st;
   const uint64_t words = num_graphs * kCkCount;
   MTRY(grow(&m->counters, &m->counters_cap, words + 1, s));
-  MTRY(grow(&m->check.part, &m->check.part_cap, L.long_rows + 1, s));
+  MTRY(grow(&m->check.part, &m->check.part_cap, 2 * L.long_rows + 2, s));
   if (m->h_counters_cap < words) {
     // the previous check's counters may still be on their way into the old buffer
     MTRY(cudaStreamSynchronize(s));
@@ -514,12 +518,12 @@ mm_status mm_validate_multi_async(mm_multi* m, uint64_t num_graphs, const mm_gra
     MTRY(cudaMallocHost(&m->h_counters, cap * sizeof(unsigned long long)));
     m->h_counters_cap = cap;
   }
-  const MultiParams M = params(m, m->check, num_graphs, L, (uint64_t)kLongRow, 1);
-  const LongRows queue{m->counters + words, reinterpret_cast<uint64_t*>(m->check.part), L.long_rows};
+  const MultiParams M = params(m, m->check, num_graphs, L, (uint64_t)kPiece, 1);
+  const LongRows queue{m->counters + words, reinterpret_cast<ulonglong2*>(m->check.part), L.long_rows};
   MTRY(cudaMemsetAsync(m->counters, 0, (words + 1) * sizeof(unsigned long long), s));
   if (L.total_vertices) {
     multi_check_kernel<<<check_grid(L.total_vertices, m->num_sms), 256, 0, s>>>(M, queue);
-    if (L.long_rows) multi_check_long_kernel<<<m->num_sms * 2, 256, 0, s>>>(M, queue);
+    if (L.long_rows) multi_check_long_kernel<<<m->num_sms * 4, 256, 0, s>>>(M, queue);
   }
   MTRY(cudaGetLastError());
   MTRY(cudaMemcpyAsync(m->h_counters, m->counters, words * sizeof(unsigned long long),
