@@ -90,7 +90,14 @@ typedef struct mm_options {
                                 layout below 6), up to 32768 for MM_HOST_MAPPED handles,
                                 whose units each start by waiting on the host link.  Batched and multi-graph calls choose
                                 from all their graphs together, down to 128.
-                                mm_skipper_static takes 0 as 2048. */
+                                mm_skipper_static takes 0 as 2048.
+                                mm_skipper walks a CSR of at most 8192 rows and
+                                32768 rows + entries in one block, its states in
+                                shared memory, when grain, blocks_per_sm and
+                                unit_order are 0 and block_threads is 0 or 512;
+                                setting one of them, timing, stats, l2_persist,
+                                stage_windows, poison_vertex or selective loads
+                                selects the sweep. */
     uint32_t block_threads;  /* sweep threads per block, multiple of 32, <= 512;
                                 0 = 512 */
     uint32_t blocks_per_sm;  /* sweep blocks per SM; 0 = the occupancy maximum of the
@@ -117,8 +124,12 @@ typedef struct mm_options {
     uint32_t l2_persist;     /* 1: L2 access-policy window (persisting) over the
                                 state array for the sweep; 0 = per-load hints only */
     uint32_t stats;          /* 1: count reads, attempts and JIT conflicts in the
-                                sweep (slower kernel instance); read back with
-                                mm_get_stats() */
+                                sweep; read back with mm_get_stats().  A slower
+                                kernel instance whose attempts are all ordered
+                                (reserve the lower id, then claim the higher), as
+                                the paper counts them; other calls try both ends
+                                of an edge at once first, so their conflicts are
+                                not these. */
     uint64_t spin_limit;     /* polls of one wait before the call fails with
                                 MM_ERR_TIMEOUT; 0 = 1 << 20 */
     uint64_t poison_vertex;  /* fault injection for tests: v + 1 leaves vertex v
@@ -485,9 +496,12 @@ mm_status mm_timing_history(mm_graph *g, mm_timing *out, uint32_t max, uint32_t 
  * grain in {2048, 8192}, status_bits in {2, 8, 32}, block_threads 512 with
  * blocks_per_sm either the 40-register or the 32-register instance's
  * occupancy, unit_order ascending or dispersed (edge-list handles: grain and
- * status_bits only) -- on this graph with CUDA events: one untimed and three
- * timed runs each, a candidate whose first timed run is already 1.5x slower
- * than the best run so far being dropped.  Every new best is checked by
+ * status_bits only), and in every layout the library's own choice (grain,
+ * blocks_per_sm and unit_order 0) where its units hold 1024 items or more or
+ * one block walks the graph (see grain) -- on this graph with CUDA events
+ * around the call: one untimed and three timed runs each, a candidate whose
+ * first timed run is already 1.5x slower than the best run so far being
+ * dropped.  Every new best is checked by
  * mm_validate (an invalid result fails the call with MM_ERR_CUDA), and the
  * fastest is written into *o; other fields of *o (symmetric, id_loads, ...)
  * are kept and apply to every candidate.  d_mate_scratch: uint32_t[n].
@@ -503,8 +517,9 @@ mm_status mm_autotune(mm_graph *g, uint32_t *d_mate_scratch, mm_options *o, void
  * {1024, 2048, 4096, 8192}, status_bits in {2, 8, 32}, block_threads 512 with
  * blocks_per_sm either the 40-register instance's or the 32-register
  * instance's occupancy (see blocks_per_sm), unit_order ascending or dispersed,
- * warps_per_graph in {0 (no cap), 4, 16} -- on this batch with CUDA
- * events: one untimed and three timed runs each, a candidate whose first timed
+ * warps_per_graph in {0 (no cap), 4, 16}, and in every layout the library's own
+ * choice, uncapped, where its units hold 1024 items or more -- on this batch
+ * with CUDA events: one untimed and three timed runs each, a candidate whose first timed
  * run is already 1.5x slower than the best run so far being dropped.  Every
  * new best is checked by the device checker (mm_validate_batched; an invalid
  * result fails the call with MM_ERR_CUDA), and the fastest is written into

@@ -1355,6 +1355,85 @@ mm_status mm_validate_batched(mm_graph* g, uint64_t num_graphs, const int64_t* d
   return MM_OK;
 }
 
+}  // extern "C"
+
+namespace {
+
+// The autotuners' race.  A candidate is run once untimed and three times timed,
+// from the stream's side (events around the whole call: a one-block pass has no
+// kernel times of its own), and dropped once 1.5x slower than the best run so
+// far; every new best is checked.
+struct Race {
+  cudaEvent_t from = nullptr, to = nullptr;
+  float best = 1e30f;
+  mm_options pick;
+  ~Race() {
+    if (from) cudaEventDestroy(from);
+    if (to) cudaEventDestroy(to);
+  }
+  mm_status open(const mm_options& o) {
+    pick = o;
+    CUDA_TRY(cudaEventCreate(&from));
+    CUDA_TRY(cudaEventCreate(&to));
+    return MM_OK;
+  }
+  // call(): enqueues the candidate and does not wait; check(v): the checker's verdict on its result
+  template <class Call, class Check>
+  mm_status run(mm_graph* g, const mm_options& c, cudaStream_t s, Call call, Check check) {
+    mm_status st;
+    float total = 0;
+    for (int rep = 0; rep < 4; ++rep) {
+      CUDA_TRY(cudaEventRecord(from, s));
+      if ((st = call()) != MM_OK) return st;
+      CUDA_TRY(cudaEventRecord(to, s));
+      if ((st = mm_sync(g, s)) != MM_OK) return st;
+      float ms = 0;
+      CUDA_TRY(cudaEventElapsedTime(&ms, from, to));
+      if (rep == 0) continue;
+      total += ms;
+      if (rep == 1 && best < 1e30f && ms > 1.5f * (best / 3.0f)) return MM_OK;
+    }
+    if (total >= best) return MM_OK;
+    mm_verdict v;
+    if ((st = check(&v)) != MM_OK) return st;
+    if (v.flags) return fail(MM_ERR_CUDA, "autotune candidate gave an invalid matching (flags 0x%x)", v.flags);
+    best = total;
+    pick.grain = c.grain;
+    pick.status_bits = c.status_bits;
+    pick.block_threads = c.block_threads;
+    pick.blocks_per_sm = c.blocks_per_sm;
+    pick.unit_order = c.unit_order;
+    pick.warps_per_graph = c.warps_per_graph;  // tuned in batched calls alone
+    return MM_OK;
+  }
+};
+
+// a tuned call's options but for what is tuned
+mm_options tuned_call(const mm_options& o, uint32_t bits) {
+  mm_options c = o;
+  c.status_bits = bits;
+  c.block_threads = kDefaultBlock;
+  c.serial = c.use_graph = c.timing = 0;
+  c.nosync = 1;
+  return c;
+}
+
+// The library's own split, occupancy and order of units are a candidate where
+// they are of the searched kind (units of 1024 items or more) or one that no
+// explicit setting asks for (one block walks the graph): a tuned call is then
+// never slower than one with the defaults.
+mm_options own_choice(const mm_options& c) {
+  mm_options d = c;
+  d.grain = d.blocks_per_sm = 0;
+  d.unit_order = MM_ORDER_AUTO;
+  return d;
+}
+constexpr uint32_t kOwnGrain = 1024;
+
+}  // namespace
+
+extern "C" {
+
 mm_status mm_autotune(mm_graph* g, uint32_t* d_mate_scratch, mm_options* o, void* cuda_stream) {
   g_err[0] = 0;
   mm_status st = check_handle(g);
@@ -1363,54 +1442,35 @@ mm_status mm_autotune(mm_graph* g, uint32_t* d_mate_scratch, mm_options* o, void
   if (g->local_ids) return fail(MM_ERR_UNSUPPORTED, "a MM_BATCH_LOCAL_IDS handle is tuned by mm_autotune_batched");
   static const uint32_t grains[] = {2048, 8192};
   static const uint32_t bits[] = {2, 8, 32};
-  const uint32_t bt = 512;
-  float best = 1e30f;
-  mm_options best_o = *o;
+  cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
+  Race race;
+  if ((st = race.open(*o)) != MM_OK) return st;
+  auto run = [&](const mm_options& c) {
+    return race.run(g, c, s, [&] { return mm_skipper(g, &c, d_mate_scratch, nullptr, 0, nullptr, s); },
+                    [&](mm_verdict* v) { return mm_validate(g, d_mate_scratch, nullptr, 0, v, s); });
+  };
+  for (uint32_t sb : bits) {
+    mm_options own = own_choice(tuned_call(*o, sb));
+    own.stats = 0;
+    Resolved r;
+    if ((st = resolve(g, &own, &r)) != MM_OK) return st;
+    if ((r.grain >= kOwnGrain || (!g->coo && chip_single(g, r, make_params(g, r, d_mate_scratch)))) &&
+        (st = run(own)) != MM_OK)
+      return st;
+  }
   for (uint32_t gr : grains)
     for (uint32_t sb : bits)
       for (int lean = 0; lean < 2; ++lean)
         for (uint32_t ord : {MM_ORDER_ASCENDING, MM_ORDER_DISPERSED}) {
           if (g->coo && (lean || ord == MM_ORDER_DISPERSED)) continue;  // edge lists: one instance, one order
-          const uint32_t bps = g->coo ? 0u : (uint32_t)sweep_blocks_per_sm((int)sb, (int)bt, lean != 0);
-          mm_options c = *o;
-          c.grain = gr;
-          c.status_bits = sb;
-          c.block_threads = bt;
-          c.blocks_per_sm = bps;
-          c.unit_order = ord;
-          c.serial = 0;
-          c.nosync = 0;
+          mm_options c = tuned_call(*o, sb);
           c.stats = 0;
-          c.timing = 1;
-          // one untimed run, then timed runs; dropped once 1.5x slower than the best run so far
-          float total = 0;
-          int reps = 0;
-          bool dropped = false;
-          for (int rep = 0; rep < 4; ++rep) {
-            if ((st = mm_skipper(g, &c, d_mate_scratch, nullptr, 0, nullptr, cuda_stream)) != MM_OK) return st;
-            mm_timing t;
-            if ((st = mm_get_timing(g, &t)) != MM_OK) return st;
-            if (rep == 0) continue;
-            total += t.total_ms;
-            ++reps;
-            if (rep == 1 && best < 1e30f && t.total_ms > 1.5f * (best / 3.0f)) {
-              dropped = true;
-              break;
-            }
-          }
-          if (dropped || reps != 3 || total >= best) continue;
-          mm_verdict v;
-          if ((st = mm_validate(g, d_mate_scratch, nullptr, 0, &v, cuda_stream)) != MM_OK) return st;
-          if (v.flags) return fail(MM_ERR_CUDA, "autotune candidate gave an invalid matching (flags 0x%x)", v.flags);
-          best = total;
-          best_o = *o;
-          best_o.grain = gr;
-          best_o.status_bits = sb;
-          best_o.block_threads = bt;
-          best_o.blocks_per_sm = bps;
-          best_o.unit_order = ord;
+          c.grain = gr;
+          c.blocks_per_sm = g->coo ? 0u : (uint32_t)sweep_blocks_per_sm((int)sb, kDefaultBlock, lean != 0);
+          c.unit_order = ord;
+          if ((st = run(c)) != MM_OK) return st;
         }
-  *o = best_o;
+  *o = race.pick;
   return MM_OK;
 }
 
@@ -1425,60 +1485,35 @@ mm_status mm_autotune_batched(mm_graph* g, uint64_t num_graphs, const int64_t* d
   static const uint32_t grains[] = {1024, 2048, 4096, 8192};
   static const uint32_t bits[] = {2, 8, 32};
   static const uint32_t wpgs[] = {0, 4, 16};
-  const uint32_t bt = 512;
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-  float best = 1e30f;
-  mm_options best_o = *o;
+  Race race;
+  if ((st = race.open(*o)) != MM_OK) return st;
+  auto run = [&](const mm_options& c) {
+    return race.run(
+        g, c, s, [&] { return mm_skipper_batched(g, num_graphs, d_vbase, d_ebase, &c, d_mate_scratch, nullptr, s); },
+        [&](mm_verdict* v) { return mm_validate_batched(g, num_graphs, d_vbase, d_ebase, d_mate_scratch, v, s); });
+  };
+  for (uint32_t sb : bits) {
+    mm_options own = own_choice(tuned_call(*o, sb));
+    own.warps_per_graph = 0;
+    Resolved r;
+    if ((st = resolve(g, &own, &r, true)) != MM_OK) return st;
+    if (r.grain >= kOwnGrain && (st = run(own)) != MM_OK) return st;
+  }
   for (uint32_t gr : grains)
     for (uint32_t sb : bits)
       for (int lean = 0; lean < 2; ++lean)
         for (uint32_t ord : {MM_ORDER_ASCENDING, MM_ORDER_DISPERSED})
-        for (uint32_t wg : wpgs) {
-        // occupancy: the blocks per SM of the 40- or the 32-register instance
-        const uint32_t bps = (uint32_t)sweep_blocks_per_sm((int)sb, (int)bt, lean != 0);
-        mm_options c = *o;
-        c.grain = gr;
-        c.status_bits = sb;
-        c.block_threads = bt;
-        c.blocks_per_sm = bps;
-        c.unit_order = ord;
-        c.warps_per_graph = wg;
-        c.serial = 0;
-        c.use_graph = 0;
-        c.nosync = 0;
-        c.timing = 1;
-        // one untimed run, one timed run; a candidate already 1.5x slower than
-        // the best per run is dropped, the others get two more timed runs
-        float total = 0;
-        int reps = 0;
-        bool dropped = false;
-        for (int rep = 0; rep < 4; ++rep) {
-          if ((st = mm_skipper_batched(g, num_graphs, d_vbase, d_ebase, &c, d_mate_scratch, nullptr, s)) != MM_OK)
-            return st;
-          mm_timing t;
-          if ((st = mm_get_timing(g, &t)) != MM_OK) return st;
-          if (rep == 0) continue;
-          total += t.total_ms;
-          ++reps;
-          if (rep == 1 && best < 1e30f && t.total_ms > 1.5f * (best / 3.0f)) {
-            dropped = true;
-            break;
+          for (uint32_t wg : wpgs) {
+            // occupancy: the blocks per SM of the 40- or the 32-register instance
+            mm_options c = tuned_call(*o, sb);
+            c.grain = gr;
+            c.blocks_per_sm = (uint32_t)sweep_blocks_per_sm((int)sb, kDefaultBlock, lean != 0);
+            c.unit_order = ord;
+            c.warps_per_graph = wg;
+            if ((st = run(c)) != MM_OK) return st;
           }
-        }
-        if (dropped || reps != 3 || total >= best) continue;
-        mm_verdict v;
-        if ((st = mm_validate_batched(g, num_graphs, d_vbase, d_ebase, d_mate_scratch, &v, s)) != MM_OK) return st;
-        if (v.flags) return fail(MM_ERR_CUDA, "autotune candidate gave an invalid matching (flags 0x%x)", v.flags);
-        best = total;
-        best_o = *o;
-        best_o.grain = gr;
-        best_o.status_bits = sb;
-        best_o.block_threads = bt;
-        best_o.blocks_per_sm = bps;
-        best_o.unit_order = ord;
-        best_o.warps_per_graph = wg;
-        }
-  *o = best_o;
+  *o = race.pick;
   return MM_OK;
 }
 
