@@ -43,6 +43,24 @@ def log(*a):
     print(*a, file=sys.stderr, flush=True)
 
 
+def compact(line: dict) -> dict:
+    """The line as it is printed: floats to eight digits, and of the side
+    measures the figures alone, to six.  How each was taken and what every layout's
+    roofline repeats (bound, peak, unit) go to the log, with all digits: with them
+    the line outgrew what keeps the last 16 KB of the output."""
+    def cut(x, side):
+        if isinstance(x, dict):
+            drop = {"how", "plain_how", "searched"} if side else set()
+            if side and "achieved" in x:
+                drop |= {"bound", "peak", "unit", "peak_kind", "kernel", "bytes_per_launch", "step_bytes_alg", "step_frac"}
+            return {k: cut(v, side) for k, v in x.items() if k not in drop}
+        if isinstance(x, list):
+            return [cut(v, side) for v in x]
+        return float(f"{x:.{6 if side else 8}g}") if isinstance(x, float) else x
+    sides = ("symmetric_option", "layouts", "side_graphs", "edge_list", "batched", "served", "cpu_skipper", "serial_mode")
+    return {k: cut(v, k in sides) for k, v in line.items()}
+
+
 def parse():
     ap = argparse.ArgumentParser(description=__doc__.splitlines()[0])
     ap.add_argument("--gpus", type=int, default=1)
@@ -377,8 +395,8 @@ def run_batched(args, skp, plain=True):
                         "warps_per_graph": tuned.warps_per_graph, "autotune_seconds": tune_s,
                         "searched": "grain {1024,2048,4096,8192} x status_bits {2,8,32} x blocks per SM "
                                     "{40-register instance, 32-register instance} (512 threads) x unit order "
-                                    "{ascending, dispersed} x warps_per_graph {0 (no cap),4,16}; every new "
-                                    "best checked"}
+                                    "{ascending, dispersed} x warps_per_graph {0 (no cap),4,16}, and the "
+                                    "library's own choice (grain 0); every new best checked"}
         for _ in range(3):
             h.batched(packed.vbase, packed.ebase, mate=mate, opts=tuned)
         lat = []
@@ -1034,7 +1052,7 @@ def run_ours(args):
 
     serial_mode = None
     if rank == 0 and world == 1 and not args.no_cpu_baseline:
-        # one GPU thread walking the CSR in SGMM order (serial mode) against SGMM
+        # one warp walking the CSR in SGMM order (serial mode) against SGMM
         # on one host core, on the ER graph of n = 100,000, m = 1,000,000
         import oracle
         import graphgen as gg
@@ -1048,10 +1066,10 @@ def run_ours(args):
                 ts.append(he.timing()["total_ms"])
         _, sgmm_s = oracle.sgmm_timed(er.offsets.numpy(), er.nbrs.numpy())
         serial_mode = {"workload": "erdos_renyi n=100000 m=1000000 (nnz 2000000)",
-                       "gpu_one_thread_ms": statistics.median(ts), "sgmm_one_core_ms": sgmm_s * 1e3,
+                       "gpu_one_warp_ms": statistics.median(ts), "sgmm_one_core_ms": sgmm_s * 1e3,
                        "ratio": statistics.median(ts) / (sgmm_s * 1e3),
-                       "how": "mm_skipper serial=1 (one GPU thread, CUDA events) vs the oracle's SGMM "
-                              "(one host core); a GPU thread is not a CPU core: this is the cost of the "
+                       "how": "mm_skipper serial=1 (one warp, CUDA events) vs the oracle's SGMM "
+                              "(one host core); a warp is not a CPU core: this is the cost of the "
                               "debug mode, not a kernel-quality figure"}
 
     batched = None
@@ -1113,7 +1131,8 @@ def run_ours(args):
     }
     h.close()
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        log("detail: " + json.dumps(line))
+        print(json.dumps(compact(line)), flush=True)
     if dist:
         dist.destroy_process_group()
     return 0
