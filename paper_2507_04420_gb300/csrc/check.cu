@@ -60,7 +60,8 @@ __device__ __forceinline__ void warp_add(unsigned long long* c, uint32_t v) {
 
 // The checker over a CSR (checkwalk.cuh): one warp per 32 consecutive vertices.
 // Bound by the latency of dependent reads (four round trips a vertex), so it
-// takes as many warps as fit without spills; reading the next group's mates and
+// takes as many warps as fit without spills (the kernels over many graphs spill at
+// that count: kCheckBlocks); reading the next group's mates and
 // row ends ahead spilled and cost 5 to 12%.  The whole check, against a
 // partition, an edge pass, an existence pass with one warp a pair and a vertex
 // pass: R-MAT 22 in 170 us (579 before), a 4096 x 4096 grid in 245 us (1645).
@@ -183,7 +184,8 @@ __global__ void validate_pairs_kernel(uint64_t n, const uint32_t* __restrict__ m
 }
 
 // ---- ordered compaction of (u, mate[u]), u < mate[u] ----
-// One pass: a block takes the next tile of 16384 vertices (a ticket keeps the
+// One pass (a single-pass scan with decoupled look-back, Merrill and Garland 2016):
+// a block takes the next tile of 16384 vertices (a ticket keeps the
 // tiles in order), counts its pairs, learns how many come before them from the
 // tiles before it -- each publishes its own count at once and the running total
 // as soon as it knows it, in one 64-bit word -- and writes them.  Bound by

@@ -38,7 +38,11 @@ constexpr int64_t kPiece = 8192;     // entries of a piece of a long row, at mos
 // piece; over many, where it also fetches each row's graph from another lane, with
 // less (40,000 rows of 3000 entries: 1560 us by warps, 690 in pieces).
 __host__ __device__ constexpr int64_t long_row(bool one) { return one ? kPiece : 2048; }
-constexpr int kCheckBlocks = 5;      // resident blocks of 256 threads an SM (4 and 6 are 5 to 10% slower)
+// Resident blocks of 256 threads an SM.  4 / 5 / 6: a 4096 x 4096 grid 211 / 186 /
+// 188 us, R-MAT 24 713 / 688 / 719.  Over many graphs, where a lane carries a graph of
+// its own and spills (176 bytes of stores in the batch kernel, 216 in the multi-graph
+// one; 56 at 4 blocks), the 4096-graph batch 474 / 492 / 496, 171 graphs 424 / 408 / 426.
+constexpr int kCheckBlocks = 5;
 
 namespace {
 
